@@ -20,7 +20,7 @@ roofline: the FP64 sweep kernel against the FP64 FMA issue rate measured on the 
          is given beside);
 vs_plain_fp64: configuration 2's comparisons -- plain FP64 cycles (which stall), FP32 inner
          cycles in FP64 / double-FP64 defect correction (time to 1e-10) -- and
-         fp32_sweep_roofline: the FP32 register wavefront kernel (4 sweeps per launch) timed alone
+         fp32_sweep_roofline: the FP32 register-tile kernel (8 sweeps per launch) timed alone
          against the measured FP32 FMA issue rate, and ff_sweep_roofline: the float-float
          FP64-accuracy sweep on the FP32 pipe beside the bit-exact FP64 sweep;
 highorder, batch, serve: configurations 3, 4 and 5 (17-point 8192^2 mixed precision to 1e-10;
@@ -184,13 +184,13 @@ class ClockSampler:
 # ----------------------------------------------------------------- traffic record
 
 KERNEL_SOURCES = ("kernels.cu", "stencil_dev.cuh", "grid_dev.cuh")
-# sources of the FP32 register wavefront kernel (temporal blocking)
-WAVE_REG_SOURCES = ("wave_reg.cu", "wave_reg_dev.cuh", "fold_dev.cuh", "grid_dev.cuh", "stencil_dev.cuh", "cj_internal.h")
-# FP32 instructions per 9-point update of the register wavefront kernel (second-difference form):
+# sources of the FP32 register-tile kernel (temporal blocking)
+RTILE_SOURCES = ("rtile.cu", "rtile_dev.cuh", "fold_dev.cuh", "grid_dev.cuh", "stencil_dev.cuh", "cj_internal.h")
+# FP32 operations per 9-point update of the register-tile kernel (second-difference form):
 # 1.25 first differences along the row (shared between neighbours) and 1 second difference, both
 # for the row entering the stencil; 1 vertical difference and 1 second difference; 1 sum of the
 # outer rows' second differences, 1 subtraction of r, 2 coefficient fmas, 1 update fma
-FP32_OPS_PER_UPDATE_WAVE_REG_9 = 9.25
+FP32_OPS_PER_UPDATE_RTILE_9 = 9.25
 # FP32 issue peak: 4 schedulers x 32 lanes per SM x 152 SMs x 2.07 GHz (FFMA/FADD issue at one
 # warp instruction per scheduler per clock)
 FP32_ISSUE_PEAK_TOPS = 4 * 32 * 152 * 2.07e9 / 1e12
@@ -439,7 +439,7 @@ def mixed_paths(cj, f, stream, fp64dd, peaks):
         k = depth if depth else 4
         out[name] = {"time_s": r["seconds"], "rel_res_l2": r["rel_res_l2"], "status": cj.cj_status_string(r["rc"]),
                      "fp32_sweeps": r["sweeps"], "outer_steps": r["cycles"], "inner_cycle": M_in,
-                     "temporal_depth": depth if depth else "auto (4 for this stencil and size unless "
+                     "temporal_depth": depth if depth else "auto (8 for this stencil and size unless "
                                                            "cj_autotune_depth recorded another)",
                      "fp32_gupdates_s": upd_s / 1e9,
                      # algorithmic bytes: one HBM round trip (read e, r; write e') per launch of k sweeps
@@ -475,15 +475,15 @@ def small_solve(cj, stream, runs: int = 5) -> dict:
 
 
 def fp32_sweep_roofline(cj, stream, peaks, launches: int = 64) -> dict:
-    """The dominant kernel of the FP32-inner paths, the register wavefront at its default depth
-    (4 sweeps per launch), timed alone with CUDA events on the launching stream over `launches`
+    """The dominant kernel of the FP32-inner paths, the register tiles at their default depth
+    (8 sweeps per launch), timed alone with CUDA events on the launching stream over `launches`
     launches on the 4096^2 grid (three 64 MB FP32 grids, more than the L2), against the FP32
     FMA issue rate measured on this GPU: it is bound by instruction issue, not by HBM."""
     import torch
     with cj.Plan(N_GRID, N_GRID, STENCIL, TOL, precision=cj.CJ_FP32_INNER) as p:
         r = torch.zeros((N_GRID, N_GRID), dtype=torch.float32, device="cuda")
         e = torch.zeros_like(r)
-        depth = 4
+        depth = 8
         cj.cj_sweeps_f32(p.handle, r, e, 0, 4 * depth, stream)
         e0 = torch.cuda.Event(enable_timing=True)
         e1 = torch.cuda.Event(enable_timing=True)
@@ -494,10 +494,10 @@ def fp32_sweep_roofline(cj, stream, peaks, launches: int = 64) -> dict:
         torch.cuda.synchronize()
     per_launch = e0.elapsed_time(e1) * 1e-3 / launches
     upd = depth * N_GRID * N_GRID
-    achieved = FP32_OPS_PER_UPDATE_WAVE_REG_9 * upd / per_launch / 1e12
-    traffic = traffic_per_launch("sweep_wave_reg_9_d4_4096", WAVE_REG_SOURCES)
+    achieved = FP32_OPS_PER_UPDATE_RTILE_9 * upd / per_launch / 1e12
+    traffic = traffic_per_launch("sweep_rtile_9_d8_4096", RTILE_SOURCES)
     peak = peaks["fp32_tfma_s"]
-    return {"kernel": "sweep_wave_reg_kernel<9,4>", "bound": "alu", "achieved": achieved,
+    return {"kernel": "sweep_rtile_kernel<9,16,8,2>", "bound": "alu", "achieved": achieved,
             "peak": peak, "unit": "TFP32op/s", "frac": achieved / peak,
             "peak_nominal": FP32_ISSUE_PEAK_TOPS, "frac_of_nominal": achieved / FP32_ISSUE_PEAK_TOPS,
             "traffic": traffic,
@@ -506,7 +506,7 @@ def fp32_sweep_roofline(cj, stream, peaks, launches: int = 64) -> dict:
             # DRAM bytes actually moved (ncu traffic per launch) per second and per update
             "dram_gbs_with_temporal_blocking": None if traffic is None else traffic / per_launch / 1e9,
             "dram_bytes_per_update": None if traffic is None else traffic / upd,
-            # algorithmic bytes: one round trip of e, r, e' (12 B per node) per launch of 4 sweeps
+            # algorithmic bytes: one round trip of e, r, e' (12 B per node) per launch of 8 sweeps
             "hbm_gbs_algorithmic": 12.0 * N_GRID * N_GRID / per_launch / 1e9,
             "peak_note": "FP32 FMA issue rate measured by cj_issue_peaks, of measured; 9.25 FP32 instructions "
                          "per 9-point update in the kernel's shared second-difference form"}

@@ -100,9 +100,9 @@ typedef struct {
                                0 = auto (the planner's choice for FP32 or FP64 inner sweeps) */
     int temporal_depth;     /* FP32-inner modes: sweeps fused per HBM round trip (temporal
                                blocking), 1..8; 0 = auto: the depth cj_autotune_depth
-                               recorded for this stencil and size class, else 4 for the
-                               5-point stencil on grids of 2^16 nodes or more and the
-                               9-point one on grids of 2^20 or more, else 1 */
+                               recorded for this stencil and size class, else the depth
+                               (up to 16; 17 points: 8) with the shortest modelled time per
+                               sweep for the grid's size */
     long long max_sweeps;   /* sweep budget of one solve; 0 = 64 cycles (CJ_JACOBI: the larger
                                of 64 intervals and 4 ln(1/tol) / kmin sweeps) */
     int method;             /* cj_method (default CJ_CJM) */
@@ -306,10 +306,9 @@ cj_status cj_sweeps_ff(cj_plan *plan, const double *f, long long ld_f, double *u
  * cj_sweeps_f32 -- apply `count` weighted FP32 sweeps e <- e + w32_n (L e - r) in place,
  * w32_n = (float) w_n of the plan's inner cycle (FP32-inner plans only), fused
  * temporal_depth at a time per launch as the solve does (bit-identical to one at a time):
- * depths 2-4 (5 and 9 points) and 2 (17 points) by the register wavefront kernel, 8 (and
- * 17-point 4) by the shared-memory wavefront kernel, 1 by the one-sweep kernel; a remainder
- * shorter than the depth, or a depth no kernel serves, runs at the largest served depth that
- * fits.  r, e: device, Ny x ld floats.  Asynchronous on `stream`.
+ * depths of 2 and more by the register-tile kernel, 1 by the one-sweep kernel; a remainder
+ * shorter than the depth runs as one launch of its own.  r, e: device, Ny x ld floats.
+ * Asynchronous on `stream`.
  */
 cj_status cj_sweeps_f32(cj_plan *plan, const float *r, long long ld_r, float *e, long long ld_e,
                         long long first, long long count, void *stream);

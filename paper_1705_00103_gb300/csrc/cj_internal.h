@@ -32,6 +32,8 @@ Grid make_grid(int Nx, int Ny, int elem_bytes);
 constexpr int kBX = 128;
 // Deepest temporal blocking of the FP32 inner sweep (sweeps per HBM round trip).
 constexpr int kTbMaxDepth = 8;
+// Most sweeps of one register-tile launch (17 points: half of it).
+constexpr int kRtMaxDepth = 16;
 struct March {
     int nbx, nby, ty;
     int blocks() const { return nbx * nby; }
@@ -170,15 +172,13 @@ cudaError_t launch_defect_dd64(const cj_plan *p, const double *uh, const double 
                                double *e_zero, cudaStream_t s);
 cudaError_t launch_correct_dd64(const cj_plan *p, double *uh, double *ul, const double *e,
                                 cudaStream_t s);
-// register wavefront temporal-blocked FP32 sweeps (wave_reg.cu): k = 2 sweeps per launch, or
-// 3 or 4 for the 5- and 9-point stencils
-int wave_reg_supported(int st, int k);
-cudaError_t launch_sweep32_wave_reg(const cj_plan *p, const float *e, const float *r, float *out,
-                                    const float *w, int k, cudaStream_t s);
-// wavefront temporal-blocked FP32 sweeps (wave.cu): k in {2, 4, 8} sweeps per launch
-int wave_depth_supported(int k);
-cudaError_t launch_sweep32_wave(const cj_plan *p, const float *e, const float *r, float *out,
-                                const float *w, int k, cudaStream_t s);
+// register-tile FP32 sweeps (rtile.cu): k sweeps per launch, 1 <= k <= kRtMaxDepth (17 points: half)
+cudaError_t launch_sweep32_rtile(const cj_plan *p, const float *e, const float *r, float *out,
+                                 const float *w, int k, cudaStream_t s);
+// sweeps per launch with the shortest modelled time per sweep, for cycles of `sweeps` sweeps
+int rtile_depth(int st, int Nx, int Ny, long long sweeps);
+// the kernels' shared-memory limits on the current device (once per plan)
+cudaError_t rtile_prepare(int st);
 cudaError_t launch_import32(const cj_plan *p, const float *src, long long ld, float *dst_pad,
                             cudaStream_t s);
 cudaError_t launch_export32(const cj_plan *p, const float *src_pad, float *dst, long long ld,

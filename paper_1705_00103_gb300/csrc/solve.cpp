@@ -373,18 +373,14 @@ cudaError_t fp32_sweeps(cj_plan *p, float **cur, float **nxt, const float *r, lo
                         long long count, cudaStream_t s, long long *launches) {
     long long n = 0;
     while (n < count) {
-        long long k = p->depth < count - n ? p->depth : count - n;
-        // the temporal-blocking kernels exist for depths 2, 3 and 4 (register wavefront; 17
-        // points: 2) and 2, 4 and 8 (wavefront strips): use the largest that fits
-        while (k > 1 && !wave_reg_supported(p->st, (int)k) && !wave_depth_supported((int)k)) --k;
+        const long long k = p->depth < count - n ? p->depth : count - n;
         cudaError_t e;
         if (k == 1) {
             e = launch_sweep32(p, *cur, r, *nxt, p->w32[(first + n) % p->M_in], s);
         } else {
-            float w[kTbMaxDepth];
+            float w[kRtMaxDepth];
             for (long long q = 0; q < k; ++q) w[q] = p->w32[(first + n + q) % p->M_in];
-            e = wave_reg_supported(p->st, (int)k) ? launch_sweep32_wave_reg(p, *cur, r, *nxt, w, (int)k, s)
-                                                   : launch_sweep32_wave(p, *cur, r, *nxt, w, (int)k, s);
+            e = launch_sweep32_rtile(p, *cur, r, *nxt, w, (int)k, s);
         }
         if (e != cudaSuccess) return e;
         float *t = *cur;
@@ -673,15 +669,12 @@ cj_status cj_plan_create(int Nx, int Ny, cj_stencil st, cj_bc bc, double tol,
             p->w32.resize(p->M_in);
             for (long long k = 0; k < p->M_in; ++k) p->w32[k] = (float)wi[k];
         }
-        // default FP32 temporal depth, from measurements (cj_sweeps_f32, Gupd/s at depth 1 / 4):
-        // 9-point 63 / 57 at 512^2, 179 / 226 at 1024^2, 510 / 545 at 2048^2, 480 / 1211 at
-        // 4096^2, 539 / 1493 at 8192^2; 5-point 16 / 18 at 256^2, 63 / 72 at 512^2 and 481 / 1413
-        // at 4096^2; 17-point depth 1 / 2: 382 / 356 at 4096^2, 422 / 408 at 8192^2.
-        // cj_autotune_depth records a measured choice per size class, which takes precedence.
-        const int tuned = tuned_depth(st, Nx, Ny);
-        const long long nodes = (long long)Nx * Ny;
-        const int dflt = (st == 5 && nodes >= (1LL << 16)) || (st == 9 && nodes >= (1LL << 20)) ? 4 : 1;
-        p->depth = o.temporal_depth ? o.temporal_depth : tuned ? tuned : dflt;
+        // FP32 temporal depth: the option, else the measured choice cj_autotune_depth recorded for
+        // the size class, else the register tiles' (rtile.cu)
+        if (p->precision == CJ_FP32_INNER || p->precision == CJ_FP32_INNER_DD) {
+            const int tuned = tuned_depth(st, Nx, Ny);
+            p->depth = o.temporal_depth ? o.temporal_depth : tuned ? tuned : rtile_depth(st, Nx, Ny, p->M_in);
+        }
         long long unit = p->precision != CJ_FP64 ? p->M_in : p->M;
         p->max_sweeps = o.max_sweeps ? o.max_sweeps : 64 * unit;
         if (p->method == CJ_JACOBI && !o.max_sweeps) {
@@ -720,6 +713,7 @@ cj_status cj_plan_create(int Nx, int Ny, cj_stencil st, cj_bc bc, double tol,
         e = dev_alloc(&p->e0, n32);
         if (e == cudaSuccess) e = dev_alloc(&p->e1, n32);
         if (e == cudaSuccess) e = dev_alloc(&p->rt, n32);
+        if (e == cudaSuccess) e = rtile_prepare(st);
     }
     if (e == cudaSuccess) e = dev_alloc(&p->partials, (size_t)3 * parts);
     if (e == cudaSuccess) e = dev_alloc(&p->red, 8);
