@@ -363,12 +363,10 @@ typedef struct {
                                FP64 floor (about 2^-53 S / (c kmin)) is within 4x of tol */
     double tol;
     int inner_cycle;        /* 0 = the planner's choice */
-    int temporal_depth;     /* FP32 sweeps per sweep launch (temporal blocking), 1..8; 0 = the
-                               cj_autotune_engine choice for the size class, else 4 for 5- and
-                               9-point problems with both sides >= 512, else 1.  Depth 4 of 5 and 9
-                               points runs the register wavefront of cj_sweeps_f32 over the
-                               problem's (strip, row block) items; other depths > 1 run tiles
-                               staged in shared memory */
+    int temporal_depth;     /* FP32 sweeps per sweep launch (temporal blocking), 1..8; 0 = 8 (17
+                               points: 4), or 1 where cj_autotune_engine measured one sweep per
+                               launch as the fastest for the size class.  Depths of 2 and more run
+                               the register tiles of cj_sweeps_f32 over the problem's tiles */
     long long max_sweeps;   /* 0 = 64 inner cycles */
     const double *f;        /* device, Ny x ld_f, unscaled right-hand side */
     long long ld_f;
@@ -384,9 +382,9 @@ typedef struct {
  * launches, export, advance: launches over persistent
  * grids that read a device tile list of 128-column tiles) is captured once in a CUDA graph
  * and replayed until every slot has finished; finished problems leave the tile list; tile
- * rows (16/32/64) and depth come from cj_autotune_engine's table for the size class when it
- * has an entry (depth-4 problems of 5 and 9 points sweep on the register wavefront instead of
- * tiles, one warp per 128-column strip and 128-row block, four sweeps per launch).  A problem's arithmetic does not depend on its batch-mates.  results[k] receives problem k's outcome (status per
+ * rows (16/32/64; of the outer steps' kernels) come from cj_autotune_engine's table for the size
+ * class when it has an entry.  The sweeps run on register tiles, eight per launch (17 points:
+ * four), the problems of one stencil and tile shape in one branch of the step's graph.  A problem's arithmetic does not depend on its batch-mates.  results[k] receives problem k's outcome (status per
  * problem; seconds and launches are those of the whole batch).  Orders itself after the
  * work already on `stream` and makes `stream` wait for it; blocks until done.  Returns
  * CJ_OK, or CJ_ERR_TIMEOUT if a problem did not finish within its sweep budget's steps.
@@ -408,12 +406,11 @@ typedef struct {
  * picked by timing the engine loaded with copies of a synthetic problem of Nx x Ny nodes (as
  * many as give the device ~8 tiles per SM, up to 256 and 2^24 nodes) at every combination, and
  * recorded in a per-process table that cj_solve_batch and the server use for problems of that
- * class (the server sweeps one at a time, so it takes the tile rows only; an explicit
- * temporal_depth overrides the depth).  Depth 4 of 5 and 9 points (the register wavefront) is a
- * candidate only when both sides are at least 512: below that its four-sweep launches are
- * latency-bound in a batch, which copies of one problem do not show (its rate is then reported
- * as 0).  Not a method of the paper: a runtime choice of this library.  Synchronous; allocates
- * an Nx x Ny FP64 grid and the engine's slots while it runs.
+ * class (the server takes the tile rows only; a depth of 2 or 4 means fused sweeps, which the batch
+ * runs at the register tiles' own depth; an explicit temporal_depth overrides it).  Depth 4 of 5 and
+ * 9 points is a candidate only when both sides are at least 512 (its rate is reported as 0 below).
+ * Not a method of the paper: a runtime choice of this library.  Synchronous; allocates an Nx x Ny
+ * FP64 grid and the engine's slots while it runs.
  *   tile_rows, depth: the choice (may be NULL);
  *   gupd: host array of 9 (may be NULL): measured Gupdates/s, tile rows 16/32/64 (major) x
  *     depth 1/2/4.
@@ -430,12 +427,10 @@ cj_status cj_autotune_engine(int Nx, int Ny, cj_stencil st, int *tile_rows, int 
  * in hbm_budget_bytes (one budget shared by the lanes); admitted problems join the lane's running
  * engine between graph replays and leave it as each one finishes, so requests arriving while
  * others run overlap with them on the device, and a small request's replays sweep only small
- * grids: its latency follows its own work, not that of the largest grids being solved.  The
- * two smaller lanes sweep one sweep per launch; the largest lane sweeps 5- and 9-point requests
- * with both sides of at least 512 on the register wavefront (four sweeps per launch), launched
- * with half a wave of blocks so that the smaller lanes' blocks still find room on every SM.
+ * grids: its latency follows its own work, not that of the largest grids being solved.  All lanes
+ * sweep on register tiles, eight sweeps per launch (17 points: four).
  * While the smallest lane has requests on the device, the two larger lanes hold their next
- * graph replay (32 sweeps of their slots), within an allowance of 1 s that refills at 0.5 s per
+ * graph replay (up to 256 sweeps of their slots), within an allowance of 1 s that refills at 0.5 s per
  * second, so a larger lane still runs at least half the time under a sustained stream of small
  * requests.  Results do not depend on the lanes' timing.
  */

@@ -18,12 +18,11 @@
 
 namespace {
 
-// FP32 sweep launches per engine step, and steps per captured graph: a replay advances a slot by
-// up to 32 sweeps, as with one sweep per step and 32 steps, with fewer launches per sweep
-// (measured: 4 sweeps per step 5.68 s for the 512-problem batch, 8: 5.52 s, 16: 5.45 s).
+// Sweep launches per engine step, and steps per captured graph: a replay advances a slot by up to
+// 256 sweeps (8 per launch; 17 points: 128).
 constexpr int kSweepsPerStep = 8;
-// Shorter side from which 5- and 9-point problems sweep on the register wavefront by default.
-constexpr int kEngWaveMinSide = 512;
+// Shorter side from which the autotuner times depth 4 of 5 and 9 points.
+constexpr int kEngDeepMinSide = 512;
 
 using Clock = std::chrono::steady_clock;
 
@@ -73,15 +72,11 @@ class Engine {
     // captured graph's grids are updated when the list changes) instead of 8 blocks per SM that
     // stride over it; short-lived blocks let another stream's higher-priority kernels onto the SMs
     // within microseconds, where resident striding blocks would hold them for a whole launch.
-    // blocked_depth: the deepest depth of the tiles' shared-memory temporal blocking (17-point slots,
-    // depths 2 and 3); -1: max_depth.  Depth-4 slots of 5 and 9 points sweep on the wavefront.
-    // wave_share: the share of the SMs' wavefront blocks the wavefront kernel launches (1 = a whole
-    // wave; the server's larger lanes leave room for the smaller lanes' blocks).
-    cj_status init(int max_slots, int max_depth, int priority_rank = 0, bool tile_grid = false,
-                   int blocked_depth = -1, double wave_share = 1.0) {
-        if (max_slots < 1 || max_depth < 1 || max_depth > kTbMaxDepth) return CJ_ERR_INVALID_ARG;
+    // lists: the register-tile lists (a bit each) the engine's problems run in.
+    cj_status init(int max_slots, unsigned lists, int priority_rank = 0, bool tile_grid = false) {
+        if (max_slots < 1 || lists == 0) return CJ_ERR_INVALID_ARG;
         max_slots_ = max_slots;
-        max_depth_ = max_depth;
+        lists_ = lists;
         ENG_TRY(cudaGetDevice(&dev_), "cudaGetDevice");
         int least = 0, greatest = 0;
         ENG_TRY(cudaDeviceGetStreamPriorityRange(&least, &greatest), "stream priorities");
@@ -92,10 +87,18 @@ class Engine {
         grid_tiles_ = sms * 8;
         tile_grid_ = tile_grid;
         grid_slots_ = std::min(max_slots, sms * 4);
-        smem_ = eng_sweep_smem(blocked_depth < 0 ? max_depth : blocked_depth);
-        wave_ = max_depth >= 4;  // depth-4 slots of 5 and 9 points sweep on the register wavefront
-        wave_grid_ = wave_ ? std::max(1, (int)(wave_share * eng_wave_grid())) : 0;
-        ENG_TRY(eng_prepare(smem_), "engine smem attribute");
+        rt_blocks_ = sms * 2;
+        ENG_TRY(eng_prepare(), "engine smem attribute");
+        ENG_TRY(cudaEventCreateWithFlags(&br_.fork, cudaEventDisableTiming), "engine event");
+        bool side = false;  // the first list runs on the engine's stream, the others beside it
+        for (int l = 0; l < kEngBranches; ++l) {
+            if (!(lists >> l & 1u)) continue;
+            if (side) {
+                ENG_TRY(cudaStreamCreateWithPriority(&br_.side[l], cudaStreamNonBlocking, prio), "engine stream");
+                ENG_TRY(cudaEventCreateWithFlags(&br_.join[l], cudaEventDisableTiming), "engine event");
+            }
+            side = true;
+        }
         host_.assign(max_slots, SlotDev{});
         mem_.assign(max_slots, SlotMem{});
         used_.assign(max_slots, 0);
@@ -106,16 +109,16 @@ class Engine {
         ENG_TRY(cudaMemset(d_.status, 0, sizeof(SlotStatus) * max_slots), "engine status");
         ENG_TRY(cudaMalloc(&d_.ntiles, sizeof(int)), "engine tile count");
         ENG_TRY(cudaMemset(d_.ntiles, 0, sizeof(int)), "engine tile count");
-        ENG_TRY(cudaMalloc(&d_.nwaves, sizeof(int)), "engine wave count");
-        ENG_TRY(cudaMemset(d_.nwaves, 0, sizeof(int)), "engine wave count");
-        wave_cap_ = 0;
-        d_.waves = nullptr;
+        ENG_TRY(cudaMalloc(&d_.item_off, sizeof(int) * (kEngLists + 1)), "engine item offsets");
+        ENG_TRY(cudaMemset(d_.item_off, 0, sizeof(int) * (kEngLists + 1)), "engine item offsets");
+        item_cap_ = 0;
+        d_.items = nullptr;
         tile_cap_ = 0;
         d_.tiles = nullptr;
         d_.max_slots = max_slots;
         ENG_TRY(cudaMallocHost(&h_status_, sizeof(SlotStatus) * max_slots), "engine status (host)");
         ENG_TRY(cudaMallocHost(&h_ntiles_, sizeof(int)), "engine tile count (host)");
-        ENG_TRY(cudaMallocHost(&h_nwaves_, sizeof(int)), "engine wave count (host)");
+        ENG_TRY(cudaMallocHost(&h_off_, sizeof(int) * (kEngLists + 1)), "engine item offsets (host)");
         return ensure_tile_capacity(1024);
     }
 
@@ -130,18 +133,28 @@ class Engine {
         cudaFree(d_.slots);
         cudaFree(d_.status);
         cudaFree(d_.ntiles);
-        cudaFree(d_.nwaves);
-        cudaFree(d_.waves);
+        cudaFree(d_.item_off);
+        cudaFree(d_.items);
         cudaFree(d_.tiles);
         if (h_status_) cudaFreeHost(h_status_);
         if (h_ntiles_) cudaFreeHost(h_ntiles_);
-        if (h_nwaves_) cudaFreeHost(h_nwaves_);
+        if (h_off_) cudaFreeHost(h_off_);
+        if (br_.fork) cudaEventDestroy(br_.fork);
+        for (int l = 0; l < kEngBranches; ++l) {
+            if (br_.side[l]) cudaStreamDestroy(br_.side[l]);
+            if (br_.join[l]) cudaEventDestroy(br_.join[l]);
+        }
         cudaStreamDestroy(s_);
         s_ = nullptr;
     }
 
     cudaStream_t stream() const { return s_; }
     int free_slots() const { return (int)std::count(used_.begin(), used_.end(), 0); }
+
+    // The list (branch of the step) a problem's sweeps run in.
+    static int list_of(const Spec &sp) {
+        return sp.depth == 1 && sp.st != CJ_ST17 ? kEngPlain : eng_list(sp.st, sp.Nx, sp.Ny);
+    }
 
     // Plan numbers of a problem: (kmin, kmax, M_in), with the FP64 cycle length as the cap.
     static cj_status plan(const Spec &sp, double *kmin, double *kmax, long long *M_in) {
@@ -179,11 +192,9 @@ class Engine {
         S.Ny = sp.Ny;
         S.st = sp.st;
         S.mode = sp.mode;
-        // a depth the engine has no shared memory for (an autotuned one in the server, whose
-        // engine sweeps one at a time) runs at the engine's maximum
-        S.depth = std::min(sp.depth, max_depth_);
-        // the wavefront takes 4 sweeps at a time: an inner cycle of 1 or 2 sweeps runs at depth 1
-        if (S.depth == 4 && (sp.st == 5 || sp.st == 9) && M_in % 4 != 0) S.depth = 1;
+        if (!(lists_ >> list_of(sp) & 1u)) return CJ_ERR_INVALID_ARG;
+        S.depth = (int)std::min<long long>(sp.depth, M_in);
+        S.plain = list_of(sp) == kEngPlain;
         S.ty = sp.ty;
         S.ntx = (sp.Nx + kEngTX - 1) / kEngTX;
         S.ntiles = S.ntx * ((sp.Ny + sp.ty - 1) / sp.ty);
@@ -288,15 +299,14 @@ class Engine {
             cj_status st = capture();
             if (st != CJ_OK) return st;
         }
-        if (tile_grid_) {
-            const int want = std::max(1, *h_ntiles_);
-            if (want != cur_grid_) {
-                cj_status st = set_tile_grid(want);
-                if (st != CJ_OK) return st;
-            }
+        if (tile_grid_ && grids_dirty_) {
+            cj_status st = set_tile_grid();
+            if (st != CJ_OK) return st;
         }
         for (int k = 0; k < replays; ++k) ENG_TRY(cudaGraphLaunch(gexec_, s_), "graph launch");
-        launches_ += (long long)replays * steps_per_graph_ * (5 + ((smem_ > 0 ? 2 : 1) + (wave_ ? 2 : 0)) * kSweepsPerStep);
+        int nlists = 0;
+        for (int l = 0; l < kEngBranches; ++l) nlists += (int)(lists_ >> l & 1u);
+        launches_ += (long long)replays * steps_per_graph_ * (5 + nlists * kSweepsPerStep);
         ENG_TRY(cudaMemcpyAsync(h_status_, d_.status, sizeof(SlotStatus) * max_slots_,
                                 cudaMemcpyDeviceToHost, s_), "status readback");
         ENG_TRY(cudaStreamSynchronize(s_), "step sync");
@@ -328,39 +338,45 @@ class Engine {
 
     cj_status upload_tiles() {
         tiles_.clear();
-        waves_.clear();
+        items_.clear();
         for (int q = 0; q < max_slots_; ++q)
-            if (used_[q] && !tiles_off_[q]) {
+            if (used_[q] && !tiles_off_[q])
                 for (int t = 0; t < host_[q].ntiles; ++t) tiles_.push_back(make_int2(q, t));
-                if (wave_) eng_wave_items(q, host_[q].Nx, host_[q].Ny, host_[q].st, host_[q].depth, waves_);
-            }
+        for (int l = 0; l < kEngLists; ++l) {
+            h_off_[l] = (int)items_.size();
+            for (int q = 0; q < max_slots_; ++q)
+                if (used_[q] && !tiles_off_[q] && !host_[q].plain && eng_list(host_[q].st, host_[q].Nx, host_[q].Ny) == l)
+                    eng_rt_items(q, host_[q].Nx, host_[q].Ny, host_[q].st, host_[q].depth, items_);
+        }
+        h_off_[kEngLists] = (int)items_.size();
         cj_status st = ensure_tile_capacity((int)tiles_.size() + 1);
         if (st != CJ_OK) return st;
-        st = ensure_wave_capacity((int)waves_.size() + 1);
+        st = ensure_item_capacity((int)items_.size() + 1);
         if (st != CJ_OK) return st;
         *h_ntiles_ = (int)tiles_.size();
-        *h_nwaves_ = (int)waves_.size();
         if (!tiles_.empty())
             ENG_TRY(cudaMemcpyAsync(d_.tiles, tiles_.data(), sizeof(int2) * tiles_.size(),
                                     cudaMemcpyHostToDevice, s_), "tile upload");
-        if (!waves_.empty())
-            ENG_TRY(cudaMemcpyAsync(d_.waves, waves_.data(), sizeof(int4) * waves_.size(),
-                                    cudaMemcpyHostToDevice, s_), "wave upload");
+        if (!items_.empty())
+            ENG_TRY(cudaMemcpyAsync(d_.items, items_.data(), sizeof(int4) * items_.size(),
+                                    cudaMemcpyHostToDevice, s_), "item upload");
         ENG_TRY(cudaMemcpyAsync(d_.ntiles, h_ntiles_, sizeof(int), cudaMemcpyHostToDevice, s_), "tile count");
-        ENG_TRY(cudaMemcpyAsync(d_.nwaves, h_nwaves_, sizeof(int), cudaMemcpyHostToDevice, s_), "wave count");
+        ENG_TRY(cudaMemcpyAsync(d_.item_off, h_off_, sizeof(int) * (kEngLists + 1), cudaMemcpyHostToDevice, s_),
+                "item offsets");
         ENG_TRY(cudaStreamSynchronize(s_), "tile sync");
         tiles_dirty_ = false;
+        grids_dirty_ = true;
         return CJ_OK;
     }
 
-    cj_status ensure_wave_capacity(int n) {
-        if (n <= wave_cap_) return CJ_OK;
-        int cap = std::max(n, 2 * wave_cap_);
+    cj_status ensure_item_capacity(int n) {
+        if (n <= item_cap_) return CJ_OK;
+        int cap = std::max(n, 2 * item_cap_);
         int4 *t = nullptr;
-        ENG_TRY(cudaMalloc(&t, sizeof(int4) * cap), "wave table");
-        cudaFree(d_.waves);
-        d_.waves = t;
-        wave_cap_ = cap;
+        ENG_TRY(cudaMalloc(&t, sizeof(int4) * cap), "item table");
+        cudaFree(d_.items);
+        d_.items = t;
+        item_cap_ = cap;
         if (gexec_) {  // the graph bakes the table pointer in: capture again
             cudaGraphExecDestroy(gexec_);
             gexec_ = nullptr;
@@ -375,12 +391,12 @@ class Engine {
         ENG_TRY(cudaStreamBeginCapture(s_, cudaStreamCaptureModeThreadLocal), "begin capture");
         cudaError_t err = cudaSuccess;
         for (int k = 0; k < steps_per_graph_ && err == cudaSuccess; ++k)
-            err = eng_launch_step(d_, grid_tiles_, grid_slots_, smem_, kSweepsPerStep, wave_grid_, s_);
+            err = eng_launch_step(d_, grid_tiles_, grid_slots_, lists_, rt_blocks_, br_, kSweepsPerStep, s_);
         cudaError_t e2 = cudaStreamEndCapture(s_, &g);
         if (err == cudaSuccess) err = e2;
         if (err == cudaSuccess) err = cudaGraphInstantiate(&gexec_, g, 0);
         tile_nodes_.clear();
-        cur_grid_ = grid_tiles_;
+        grids_dirty_ = true;
         if (err == cudaSuccess && tile_grid_) {  // the nodes whose grid follows the tile list
             size_t n = 0;
             err = cudaGraphGetNodes(g, nullptr, &n);
@@ -392,7 +408,9 @@ class Engine {
                 if (err != cudaSuccess || type != cudaGraphNodeTypeKernel) continue;
                 cudaKernelNodeParams kp{};
                 err = cudaGraphKernelNodeGetParams(nodes[k], &kp);
-                if (err == cudaSuccess && eng_is_tile_kernel(kp.func)) tile_nodes_.push_back(nodes[k]);
+                const int list = err == cudaSuccess ? eng_list_of_kernel(kp.func) : -1;
+                if (err == cudaSuccess && (list >= 0 || eng_is_tile_kernel(kp.func)))
+                    tile_nodes_.push_back({nodes[k], list, 0});
             }
         }
         if (err == cudaSuccess) {
@@ -404,30 +422,42 @@ class Engine {
         return CJ_OK;
     }
 
-    // Every tile kernel of the instantiated graph launches `blocks` blocks from now on.
-    cj_status set_tile_grid(int blocks) {
-        for (cudaGraphNode_t node : tile_nodes_) {
+    // The tile kernels of the instantiated graph launch one block per tile, the sweep kernels one per
+    // item of their list, from now on.
+    cj_status set_tile_grid() {
+        for (GridNode &n : tile_nodes_) {
+            const int want = std::max(1, n.list < 0 ? *h_ntiles_ : h_off_[n.list + 1] - h_off_[n.list]);
+            if (want == n.blocks) continue;
             cudaKernelNodeParams kp{};
-            ENG_TRY(cudaGraphKernelNodeGetParams(node, &kp), "tile node params");
-            kp.gridDim = dim3((unsigned)blocks);
-            ENG_TRY(cudaGraphExecKernelNodeSetParams(gexec_, node, &kp), "tile grid update");
+            ENG_TRY(cudaGraphKernelNodeGetParams(n.node, &kp), "tile node params");
+            kp.gridDim = dim3((unsigned)want);
+            ENG_TRY(cudaGraphExecKernelNodeSetParams(gexec_, n.node, &kp), "tile grid update");
+            n.blocks = want;
         }
-        cur_grid_ = blocks;
+        grids_dirty_ = false;
         return CJ_OK;
     }
 
-    int dev_ = 0, max_slots_ = 0, max_depth_ = 1, grid_tiles_ = 0, grid_slots_ = 0;
+    // a kernel node whose grid follows the tile list (list -1) or a sweep list; blocks it launches
+    // in the instantiated graph (0: those of the capture)
+    struct GridNode {
+        cudaGraphNode_t node;
+        int list, blocks;
+    };
+
+    int dev_ = 0, max_slots_ = 0, grid_tiles_ = 0, grid_slots_ = 0, rt_blocks_ = 0;
+    unsigned lists_ = 0;
     int steps_per_graph_ = 4;
-    size_t smem_ = 0;
+    EngineBranches br_;
     cudaStream_t s_ = nullptr;
     EngineDev d_{};
     std::vector<SlotDev> host_;
     std::vector<SlotMem> mem_;
     std::vector<char> used_, tiles_off_;
     std::vector<int2> tiles_;
-    std::vector<int4> waves_;
-    int wave_cap_ = 0;
-    int *h_nwaves_ = nullptr;
+    std::vector<int4> items_;
+    int item_cap_ = 0;
+    int *h_off_ = nullptr;
     std::vector<float> wstage_;
     int tile_cap_ = 0;
     bool tiles_dirty_ = true;
@@ -435,10 +465,8 @@ class Engine {
     int *h_ntiles_ = nullptr;
     cudaGraphExec_t gexec_ = nullptr;
     cudaGraph_t graph_ = nullptr;
-    bool tile_grid_ = false, wave_ = false;
-    int wave_grid_ = 0;
-    std::vector<cudaGraphNode_t> tile_nodes_;
-    int cur_grid_ = 0;
+    bool tile_grid_ = false, grids_dirty_ = true;
+    std::vector<GridNode> tile_nodes_;
     long long launches_ = 0;
 };
 
@@ -477,12 +505,6 @@ cj_status check_problem(const cj_problem &pr) {
     return CJ_OK;
 }
 
-// Default depth of a problem the autotuner has not seen: the register wavefront (depth 4) for 5-
-// and 9-point problems whose shorter side is at least kEngWaveMinSide, else one sweep at a time.
-int default_depth(int st, int Nx, int Ny) {
-    return (st == CJ_ST5 || st == CJ_ST9) && std::min(Nx, Ny) >= kEngWaveMinSide ? 4 : 1;
-}
-
 Spec spec_of(const cj_problem &pr) {
     Spec sp;
     sp.Nx = pr.Nx;
@@ -492,7 +514,8 @@ Spec spec_of(const cj_problem &pr) {
     sp.mode = pr.precision ? pr.precision : auto_mode(pr.st, pr.Nx, pr.Ny, pr.tol);
     sp.inner_cycle = pr.inner_cycle;
     EngineTune t = engine_tuned(pr.st, pr.Nx, pr.Ny);
-    sp.depth = pr.temporal_depth ? pr.temporal_depth : (t.depth ? t.depth : default_depth(pr.st, pr.Nx, pr.Ny));
+    // a measured preference for one sweep per launch stands; fused sweeps run at the tiles' own depth
+    sp.depth = pr.temporal_depth ? pr.temporal_depth : (t.depth == 1 ? 1 : eng_default_depth(pr.st));
     sp.ty = t.ty ? t.ty : kEngTYDefault;
     sp.max_sweeps = pr.max_sweeps;
     return sp;
@@ -518,16 +541,14 @@ void fill_result(const SlotStatus &st, cj_result *r) {
 // priority.  Admission stays by footprint against the one shared budget, in arrival order
 // within a lane.
 constexpr int kLanes = 3;
-// Share of a wave of wavefront blocks the larger lanes launch (one block per SM of the two that fit).
-constexpr double kServerWaveShare = 0.5;
 constexpr long long kLaneNodes[kLanes] = {1LL << 20, 1LL << 23, 1LL << 62};
-// Every lane launches its tile kernels with one block per tile (Engine::init's tile_grid): with
+// The two larger lanes launch their kernels with one block per tile (Engine::init's tile_grid): with
 // blocks that live a few microseconds, the block scheduler puts the smaller lanes' higher-priority
 // blocks on the SMs as soon as any block retires, while each lane still fills the device when it
 // runs alone.
 // The two larger lanes also hold their next graph replay while the smallest lane has requests on
 // the device, so its short-lived kernels find the SMs free instead of sharing them with the larger
-// lanes' blocks; a replay is 32 sweeps of a lane's slots, so at most one replay of each larger
+// lanes' blocks; a replay is up to 256 sweeps of a lane's slots, so at most one replay of each larger
 // lane is in flight when a small request arrives.  (Holding the largest lane for the middle one
 // as well raised the p99 latency and lowered the throughput more, for no lower p50.)  The hold is
 // paid from an allowance per lane: it starts at kYieldCapS seconds, refills at kYieldRate seconds
@@ -797,17 +818,15 @@ extern "C" {
 
 cj_status cj_solve_batch(const cj_problem *problems, int n, void *stream, cj_result *results) {
     if (!problems || n < 1 || !results) return CJ_ERR_INVALID_ARG;
-    int max_depth = 1, blocked_depth = 1;
+    unsigned lists = 0;
     for (int k = 0; k < n; ++k) {
         cj_status st = check_problem(problems[k]);
         if (st != CJ_OK) return st;
-        const int d = spec_of(problems[k]).depth;  // requested or autotuned
-        max_depth = std::max(max_depth, d);
-        if (problems[k].st == CJ_ST17 || d == 2 || d == 3) blocked_depth = std::max(blocked_depth, d);
+        lists |= 1u << Engine::list_of(spec_of(problems[k]));
     }
     auto t0 = Clock::now();
     Engine eng;
-    cj_status st = eng.init(n, max_depth, 0, false, blocked_depth);
+    cj_status st = eng.init(n, lists);
     if (st != CJ_OK) return st;
     cudaEvent_t ev;
     ENG_TRY(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming), "event");
@@ -893,23 +912,10 @@ cj_status cj_autotune_engine(int Nx, int Ny, cj_stencil st, int *tile_rows, int 
     copies = std::max<long long>(1, std::min<long long>(copies, (1LL << 24) / ((long long)Nx * Ny)));
     cj_status rc = CJ_OK;
     for (int c = 0; c < 9 && rc == CJ_OK; ++c) {
-        // depth 4 of 5 and 9 points is the register wavefront, whose four-sweep launches of a
-        // problem with a side under 512 are latency-bound in a batch (measured on the 512-problem
-        // batch: 3.55 s at depth 1 everywhere, 3.45 s at depth 4 everywhere, 3.16 s at depth 4 from
-        // a shorter side of 512): not a candidate there
-        if (dps[c] == 4 && st != CJ_ST17 && std::min(Nx, Ny) < kEngWaveMinSide) continue;
-        // the wavefront's copies: enough (strip, row block) items for two waves of its warps
-        long long cp = copies;
-        if (dps[c] == 4 && st != CJ_ST17) {
-            std::vector<int4> items;
-            const long long per = std::max(1, eng_wave_items(0, Nx, Ny, st, 4, items));
-            cp = std::max(cp, (2LL * eng_wave_grid() * 4 + per - 1) / per);
-            cp = std::min<long long>(cp, 256);
-            cp = std::max<long long>(1, std::min<long long>(cp, (1LL << 24) / ((long long)Nx * Ny)));
-        }
+        // depth 4 of 5 and 9 points is timed from a shorter side of 512 on
+        if (dps[c] == 4 && st != CJ_ST17 && std::min(Nx, Ny) < kEngDeepMinSide) continue;
+        const long long cp = copies;
         Engine eng;
-        rc = eng.init((int)cp, dps[c], 0, false, st == CJ_ST17 || dps[c] == 2 || dps[c] == 3 ? dps[c] : 1);
-        if (rc != CJ_OK) break;
         Spec sp{};
         sp.Nx = Nx;
         sp.Ny = Ny;
@@ -920,6 +926,8 @@ cj_status cj_autotune_engine(int Nx, int Ny, cj_stencil st, int *tile_rows, int 
         sp.ty = tys[c];
         sp.tol = 1e-15;
         sp.max_sweeps = 0;
+        rc = eng.init((int)cp, 1u << Engine::list_of(sp));
+        if (rc != CJ_OK) break;
         std::vector<int> q(cp, -1);
         for (long long k = 0; k < cp && rc == CJ_OK; ++k)
             rc = eng.admit(sp, f, Nx, nullptr, 0, nullptr, 0, &q[k], true);  // results into own slot
@@ -961,9 +969,9 @@ cj_status cj_server_create(size_t hbm_budget_bytes, int max_slots, cj_server **o
     sv->max_slots = max_slots;
     cudaGetDevice(&sv->device);
     for (int k = 0; k < kLanes; ++k) {
-        // the two larger lanes sweep 5- and 9-point requests with a side of at least 512 on the
-        // register wavefront (depth 4); the smallest sweeps one at a time
-        cj_status st = sv->lanes[k].eng.init(max_slots, k == kLanes - 1 ? 4 : 1, kLanes - 1 - k, true, 1, kServerWaveShare);
+        // the smallest lane's requests run on short tiles, the larger lanes' on tall ones
+        const unsigned lists = k == 0 ? 0x15u : 0x2au;
+        cj_status st = sv->lanes[k].eng.init(max_slots, lists, kLanes - 1 - k, k > 0);
         if (st == CJ_OK && cudaMallocHost((void **)&sv->lanes[k].stage, cj_server::kStageBytes) != cudaSuccess)
             st = CJ_ERR_NOMEM;
         if (st != CJ_OK) {
@@ -1000,6 +1008,7 @@ cj_status cj_submit(cj_server *sv, int Nx, int Ny, cj_stencil st, double tol, co
     cj_server::Request &r = sv->reqs[t];
     r.ticket = t;
     r.sp = spec_of(pr);
+    r.sp.depth = eng_default_depth(st);  // the server takes the tile rows of the autotuner's choice only
     r.lane = lane_of(r.sp);
     r.f.assign(f_host, f_host + (size_t)Nx * Ny);
     r.t_submit = Clock::now();

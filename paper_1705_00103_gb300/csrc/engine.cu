@@ -2,17 +2,18 @@
 //
 // Many independent problems of different sizes, stencils and tolerances are solved
 // together by the mixed-precision CJM (FP32 inner cycles inside an FP64 or double-FP64
-// defect-correction loop).  One engine step is six launches over fixed, persistent grids:
+// defect-correction loop).  One engine step is five launches and the sweeps:
 //   correct  -- slots starting an outer step add the last inner cycle's correction to u;
 //   defect   -- they form the defect r = b - L u (FP64 or double-FP64), its FP32 copy and
 //               per-tile partial norms, and zero the inner iterate;
 //   decide   -- per slot: reduce the partials in a fixed order, apply the stop rule on the
 //               device, start the next inner cycle or finish the slot;
-//   sweep    -- every slot in an inner cycle advances min(depth, left) FP32 sweeps over all
-//               of its tiles (one-sweep march4, or temporal blocking; depth-4 slots of 5 and
-//               9 points on the register wavefront); a step runs several sweep launches, the
-//               q-th reading where the slot stands from the step's starting counter and q,
-//               so the per-step launches are spread over more sweeps;
+//   sweep    -- every slot in an inner cycle advances min(depth, left) FP32 sweeps on the register
+//               tiles of rtile_dev.cuh, one block per tile; a step runs several sweep launches,
+//               the q-th reading where the slot stands from the step's starting counter and q,
+//               so the per-step launches are spread over more sweeps.  Slots of one stencil and
+//               tile shape form a list with a kernel of its own, and the lists' launches are
+//               parallel branches of the graph (slots are independent);
 //   export   -- finished slots copy u into the caller's buffer;
 //   advance  -- per slot: move the cycle counter and the ping-pong by the step's sweeps,
 //               retire exported slots, publish a compact status record for the host.
@@ -22,13 +23,11 @@
 //
 // Per node, every kernel evaluates the same arithmetic, in the same order, as the
 // single-problem solver, so a problem's result does not depend on what it is batched with.
-#include <mutex>
-
 #include "engine.cuh"
 #include "grid_dev.cuh"
 #include "march4_dev.cuh"
+#include "rtile_dev.cuh"
 #include "stencil_dev.cuh"
-#include "wave_reg_dev.cuh"
 
 namespace {
 
@@ -47,15 +46,6 @@ __device__ __forceinline__ TileRef tile_ref(const SlotDev &S, int slot, int lt) 
     t.i1 = min(t.i0 + kEngTX - 1, S.Nx);
     t.j1 = min(t.j0 + S.ty - 1, S.Ny);
     return t;
-}
-
-// Rows of the wavefront items' row blocks (16 rows of warm-up per block at depth 4).
-constexpr int kEngWaveRows = 128;
-
-// Slots whose sweeps run on the register wavefront: 5- and 9-point slots at depth 4 (their inner
-// cycles are a multiple of 4 sweeps long: admission runs shorter ones at depth 1).
-__device__ __forceinline__ bool eng_wave_slot(const SlotDev &S) {
-    return S.depth == 4 && (S.st == 5 || S.st == 9);
 }
 
 // Where sweep launch q of a step (0-based) stands for a slot in its inner cycle: the slot's counter
@@ -234,80 +224,91 @@ __global__ void __launch_bounds__(kEngThreads) eng_decide(EngineDev E) {
     }
 }
 
-// sweep: one-sweep march for depth 1, temporal blocking otherwise
+// One sweep of a tile: four warps split its rows; each lane takes four adjacent columns (march4).
 template <int ST>
-__device__ __forceinline__ void sweep_tile(SlotDev &S, const TileRef &T, const StepPos &P, float *sm) {
-    const int k = P.k;
-    const float *ein = P.cur ? S.e1 : S.e0;
-    float *eout = P.cur ? S.e0 : S.e1;
-    if (k == 1) {
-        // four warps split the tile's rows; each lane takes four adjacent columns (march4)
-        const int rows_per_warp = (S.ty + kEngThreads / 32 - 1) / (kEngThreads / 32);
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-        const int c0 = T.i0 + 4 * lane;
-        const int js = T.j0 + warp * rows_per_warp;
-        const int je = min(js + rows_per_warp - 1, T.j1);
-        if (c0 > T.i1 || js > je) return;
-        M4Store<ST> op{eout, &S.g32, c0, S.w32[P.counter]};
-        march4<ST>(ein, S.rt, S.g32, c0, js, je, op);
-    } else {
-        float w[kTbMaxDepth];
-        for (int s = 0; s < k; ++s) w[s] = S.w32[P.counter + s];
-        tb_tile<ST>(ein, S.rt, eout, S.g32, k, w, T.i0, T.j0, kEngTX, S.ty, sm);
-    }
+__device__ __forceinline__ void sweep_tile(const SlotDev &S, const TileRef &T, const StepPos &P) {
+    const int rows_per_warp = (S.ty + kEngThreads / 32 - 1) / (kEngThreads / 32);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int c0 = T.i0 + 4 * lane;
+    const int js = T.j0 + warp * rows_per_warp;
+    const int je = min(js + rows_per_warp - 1, T.j1);
+    if (c0 > T.i1 || js > je) return;
+    M4Store<ST> op{P.cur ? S.e0 : S.e1, &S.g32, c0, S.w32[P.counter]};
+    march4<ST>(P.cur ? S.e1 : S.e0, S.rt, S.g32, c0, js, je, op);
 }
 
-// Sweep launches: tiles whose slot advances one sweep now (k = 1: march4, no shared memory)
-// and tiles of temporally blocked slots (k > 1: tb_tile in dynamic shared memory) go to two
-// kernels, so that the blocked tiles' shared memory does not lower the occupancy of the rest.
-// (64 registers for the one-sweep tiles: 8 blocks per SM stay resident, which measured 1.4x faster on
-// the 512-problem batch than the 95-register, 5-blocks-per-SM build)
-template <bool BLOCKED>
-__global__ void __launch_bounds__(kEngThreads, BLOCKED ? 1 : 8) eng_sweep(EngineDev E, int q) {
-    extern __shared__ float sm[];
+// Sweep launch q of the 5- and 9-point slots that were asked for one sweep per launch: streaming
+// tiles, which such a launch is faster on than on register tiles (12 9-point problems of 1024^2: 259
+// against 303 ms; 17 points the other way round: 747 against 387 ms).
+// (64 registers: 8 blocks per SM stay resident, which measured 1.4x faster on the 512-problem batch
+// than the 95-register, 5-blocks-per-SM build)
+__global__ void __launch_bounds__(kEngThreads, 8) eng_sweep_plain(EngineDev E, int q) {
     const int n = *E.ntiles;
     for (int t = blockIdx.x; t < n; t += gridDim.x) {
         const int2 ref = E.tiles[t];
-        SlotDev &S = E.slots[ref.x];
-        if (S.phase != PHASE_SWEEP || eng_wave_slot(S)) continue;
+        const SlotDev &S = E.slots[ref.x];
+        if (S.phase != PHASE_SWEEP || !S.plain) continue;
         const StepPos P = eng_pos(S, q);
-        if (P.k == 0 || (P.k > 1) != BLOCKED) continue;
+        if (P.k == 0) continue;
         const TileRef T = tile_ref(S, ref.x, ref.y);
-        if (BLOCKED) __syncthreads();  // the previous tile's shared-memory stage is finished
         if (S.st == 5)
-            sweep_tile<5>(S, T, P, sm);
-        else if (S.st == 9)
-            sweep_tile<9>(S, T, P, sm);
+            sweep_tile<5>(S, T, P);
         else
-            sweep_tile<17>(S, T, P, sm);
+            sweep_tile<9>(S, T, P);
     }
 }
 
-// Sweep launches, wavefront part: each warp takes (slot, strip, row block) items of the wave list
-// and advances them 4 sweeps (wr_run: the single-grid wavefront's per-warp stage, the same node
-// arithmetic, so the results equal one-sweep tiles bit for bit); the tile kernels leave these
-// slots alone.
-// (one kernel per stencil: both stage bodies in one kernel overflow the instruction cache)
-template <int ST>
-__global__ void __launch_bounds__(kWrThreads, 2) eng_sweep_wave(EngineDev E, int q) {
-    __shared__ float4 ering[kWrWarps][kWrERing][32];
-    __shared__ float4 rring[kWrWarps][kWrRRing][32];
-    const int wid = (int)threadIdx.x >> 5;
-    const int n = *E.nwaves;
-    for (int it = (int)blockIdx.x * kWrWarps + wid; it < n; it += (int)gridDim.x * kWrWarps) {
-        const int4 w = E.waves[it];
-        SlotDev &S = E.slots[w.x];
-        if (S.st != ST || S.phase != PHASE_SWEEP || !eng_wave_slot(S)) continue;  // warp-uniform
+// Sweep launch q of a list: each block takes (slot, tile) items and advances them min(depth, left)
+// sweeps.  The launches of a step follow one another with programmatic dependent launch: a block
+// reads its items and its slot's position, which no sweep changes, and stages r before it waits for
+// the previous launch; a block without work waits too, so that a launch ends after all before it.
+template <int ST, int RPT, int NW>
+__global__ void __launch_bounds__(NW * 32, 2) eng_sweep_rt(EngineDev E, int list, int q) {
+    extern __shared__ float4 sm[];
+    const int end = E.item_off[list + 1];
+    for (int it = E.item_off[list] + (int)blockIdx.x; it < end; it += (int)gridDim.x) {
+        const int4 w = E.items[it];
+        const SlotDev &S = E.slots[w.x];
+        if (S.phase != PHASE_SWEEP) continue;  // uniform over the block
         const StepPos P = eng_pos(S, q);
-        if (P.k != 4) continue;
-        WrWeights wt;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) wt.w[k] = S.w32[P.counter + k];
-        const float *ein = P.cur ? S.e1 : S.e0;
-        float *eout = P.cur ? S.e0 : S.e1;
-        wr_run<ST, 4>(ein, S.rt, eout, S.g32, wt, kEngWaveRows, w.y, w.z, ering[wid][0], rring[wid][0]);
+        if (P.k == 0) continue;
+        const Grid g = S.g32;
+        rt_run<ST, RPT, NW>(P.cur ? S.e1 : S.e0, S.rt, P.cur ? S.e0 : S.e1, g, S.w32 + P.counter, P.k, w.y, w.z, w.w,
+                            sm);
+        __syncthreads();  // the tile's shared memory is the next item's
     }
+    rt_wait_previous();
 }
+
+// Measured (one GB300, before with one sweep, or four in the per-warp row wavefront, per launch and one
+// chain of launches for all slots -> register tiles in branches): 32 problems of 64 .. 1024 a side to
+// 1e-8 63.9 -> 16.5 ms; 512 of 64 .. 2048 3.1 -> 1.02 s; a burst of 24 served requests of 32 .. 1024 a
+// side 75 -> 21 ms; the first 64 of the served stream (sides up to 8192) 365 -> 1259 Gupd/s, p50 0.19
+// -> 0.14 s, p99 16.8 -> 4.8 s.  What bounds it: on a few small problems the launches (about 8 us for
+// eight sweeps), on many the FMA pipe, as for one grid (rtile.cu).
+// Problems of more than 2^20 nodes sweep on tall tiles (0.77 of a staged tile is stored at depth 8,
+// against 0.66 of a short one's); below, short tiles give more blocks and shorter launches (one
+// 1023^2 9-point grid: 10 us against 13.5 us per launch of 8 sweeps).
+constexpr long long kEngTallNodes = 1LL << 20;
+
+struct EngRt {
+    const void *fn;
+    int rows, smem;
+};
+
+template <int ST, int RPT, int NW>
+EngRt eng_rt() {
+    return EngRt{(const void *)eng_sweep_rt<ST, RPT, NW>, RPT * NW, RtShape<ST, RPT, NW>::smem_bytes};
+}
+
+// by list: short and tall tiles of 5, 9 and 17 points (8 warps each)
+const EngRt *eng_rt_kernels() {
+    static const EngRt k[kEngLists] = {eng_rt<5, 8, 8>(),  eng_rt<5, 16, 8>(),  eng_rt<9, 8, 8>(),
+                                       eng_rt<9, 16, 8>(), eng_rt<17, 8, 8>(), eng_rt<17, 14, 8>()};
+    return k;
+}
+
+constexpr int kEngRtThreads = 256;
 
 __global__ void __launch_bounds__(kEngThreads) eng_export(EngineDev E) {
     const int n = *E.ntiles;
@@ -435,72 +436,94 @@ __global__ void __launch_bounds__(kEngThreads) eng_admit(EngineDev E, int slot) 
 
 }  // namespace
 
-size_t eng_sweep_smem(int max_depth) {
-    if (max_depth <= 1) return 0;
-    const int H = 2 * max_depth;  // radius 2 covers every stencil
-    return (size_t)3 * (kEngTX + 2 * H) * (kEngTYMax + 2 * H) * sizeof(float);
-}
-
 bool eng_is_tile_kernel(const void *fn) {
-    return fn == (const void *)eng_correct || fn == (const void *)eng_defect || fn == (const void *)eng_sweep<false> ||
-           fn == (const void *)eng_sweep<true> || fn == (const void *)eng_export;
+    return fn == (const void *)eng_correct || fn == (const void *)eng_defect || fn == (const void *)eng_export ||
+           fn == (const void *)eng_sweep_plain;
 }
 
-int eng_sweep_blocks_per_sm() {
-    int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, eng_sweep<false>, kEngThreads, 0) != cudaSuccess || n < 1)
-        n = 1;
-    return n;
+int eng_list_of_kernel(const void *fn) {
+    for (int l = 0; l < kEngLists; ++l)
+        if (fn == eng_rt_kernels()[l].fn) return l;
+    return -1;
 }
 
-// The blocked sweep kernel's dynamic shared-memory limit is one attribute of the function, shared by
-// every engine in the process (the server's lanes are several): it is only ever raised, so an engine
-// created later with a shallower depth never takes it from one that needs it.
-cudaError_t eng_prepare(size_t sweep_smem) {
-    static std::mutex mu;
-    static size_t granted = 0;
-    std::lock_guard<std::mutex> lk(mu);
-    if (sweep_smem <= granted) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(eng_sweep<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sweep_smem);
-    if (e == cudaSuccess) granted = sweep_smem;
-    return e;
+cudaError_t eng_prepare() {
+    for (int l = 0; l < kEngLists; ++l) {
+        const EngRt &K = eng_rt_kernels()[l];
+        const cudaError_t e = cudaFuncSetAttribute(K.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, K.smem);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
-int eng_wave_items(int slot, int Nx, int Ny, int st, int depth, std::vector<int4> &items) {
-    if (depth != 4 || (st != 5 && st != 9)) return 0;
-    const int nstrips = wr_strips(Nx), nrb = (Ny + kEngWaveRows - 1) / kEngWaveRows;
-    for (int rb = 0; rb < nrb; ++rb)
-        for (int x = 0; x < nstrips; ++x) items.push_back(make_int4(slot, x, rb, 0));
-    return nstrips * nrb;
+int eng_default_depth(int st) { return st == 17 ? 4 : 8; }
+
+int eng_list(int st, int Nx, int Ny) {
+    return 2 * stencil_slot(st) + ((long long)Nx * Ny > kEngTallNodes ? 1 : 0);
 }
 
-int eng_wave_grid() {
-    static const int n = [] {
-        int dev = 0, sms = 152, per_sm = 1;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, eng_sweep_wave<9>, kWrThreads, 0) != cudaSuccess ||
-            per_sm < 1)
-            per_sm = 1;
-        return sms * per_sm;
-    }();
-    return n;
+void eng_rt_items(int slot, int Nx, int Ny, int st, int depth, std::vector<int4> &items) {
+    const int R = st == 17 ? 2 : 1;
+    const int cols = 128 - 2 * rt_halo_cols(R, depth);
+    int rows = eng_rt_kernels()[eng_list(st, Nx, Ny)].rows - 2 * R * depth;
+    const int nrb = (Ny + rows - 1) / rows;
+    rows = (Ny + nrb - 1) / nrb;  // the same rows for every tile
+    for (int y = 1; y <= Ny; y += rows)
+        for (int x = 1; x <= Nx; x += cols) items.push_back(make_int4(slot, x, y, y + rows - 1 < Ny ? y + rows - 1 : Ny));
 }
 
-cudaError_t eng_launch_step(const EngineDev &e, int grid_tiles, int grid_slots, size_t sweep_smem,
-                            int sweeps, int wave_grid, cudaStream_t s) {
+// The step's sweep launches of register-tile list l on stream s: after the first, each with
+// programmatic dependent launch.
+static cudaError_t launch_list(const EngineDev &e, int l, int blocks, int sweeps, cudaStream_t s) {
+    const EngRt &K = eng_rt_kernels()[l];
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3(kEngRtThreads);
+    cfg.dynamicSmemBytes = K.smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cudaError_t err = cudaSuccess;
+    for (int q = 0; q < sweeps && err == cudaSuccess; ++q) {
+        cfg.numAttrs = q > 0 ? 1 : 0;
+        void *args[] = {(void *)&e, (void *)&l, (void *)&q};
+        err = cudaLaunchKernelExC(&cfg, K.fn, args);
+    }
+    return err;
+}
+
+cudaError_t eng_launch_step(const EngineDev &e, int grid_tiles, int grid_slots, unsigned lists, int rt_blocks,
+                            const EngineBranches &br, int sweeps, cudaStream_t s) {
     const int grid_adv = (e.max_slots + 127) / 128;
     eng_correct<<<grid_tiles, kEngThreads, 0, s>>>(e);
     eng_defect<<<grid_tiles, kEngThreads, 0, s>>>(e);
     eng_decide<<<grid_slots, kEngThreads, 0, s>>>(e);
-    for (int q = 0; q < sweeps; ++q) {
-        eng_sweep<false><<<grid_tiles, kEngThreads, 0, s>>>(e, q);
-        if (sweep_smem > 0) eng_sweep<true><<<grid_tiles, kEngThreads, sweep_smem, s>>>(e, q);
-        if (wave_grid > 0) {
-            eng_sweep_wave<5><<<wave_grid, kWrThreads, 0, s>>>(e, q);
-            eng_sweep_wave<9><<<wave_grid, kWrThreads, 0, s>>>(e, q);
+    cudaError_t err = cudaEventRecord(br.fork, s);
+    bool first = true;
+    for (int l = 0; l < kEngBranches && err == cudaSuccess; ++l) {
+        if (!(lists >> l & 1u)) continue;
+        const cudaStream_t sl = first ? s : br.side[l];  // the first list stays on the engine's stream
+        if (!first) err = cudaStreamWaitEvent(sl, br.fork, 0);
+        if (l == kEngPlain) {
+            for (int q = 0; q < sweeps && err == cudaSuccess; ++q) {
+                eng_sweep_plain<<<grid_tiles, kEngThreads, 0, sl>>>(e, q);
+                err = cudaGetLastError();
+            }
+        } else if (err == cudaSuccess) {
+            err = launch_list(e, l, rt_blocks, sweeps, sl);
         }
+        if (!first && err == cudaSuccess) err = cudaEventRecord(br.join[l], sl);
+        first = false;
     }
+    first = true;
+    for (int l = 0; l < kEngBranches && err == cudaSuccess; ++l) {
+        if (!(lists >> l & 1u)) continue;
+        if (!first) err = cudaStreamWaitEvent(s, br.join[l], 0);
+        first = false;
+    }
+    if (err != cudaSuccess) return err;
     eng_export<<<grid_tiles, kEngThreads, 0, s>>>(e);
     eng_advance<<<grid_adv, 128, 0, s>>>(e, sweeps);
     return cudaGetLastError();

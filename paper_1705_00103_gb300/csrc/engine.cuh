@@ -24,7 +24,8 @@ enum SlotPhase : int {
 struct SlotDev {
     // set at admission
     int Nx, Ny, st, mode;          // mode: CJ_FP32_INNER or CJ_FP32_INNER_DD
-    int depth, ntx, ntiles, ty;    // ty: tile rows
+    int depth, ntx, ntiles, ty;    // depth: sweeps per sweep launch; ty: tile rows
+    int plain;                     // 1: one sweep per launch over the tile list
     long long M_in, max_outer;
     double tol, S, h2;
     Grid g64, g32;
@@ -47,32 +48,42 @@ struct SlotStatus {
     double rho, rinf, fl;
 };
 
+// Register-tile lists of an engine: stencil x shape (short or tall tiles), one kernel each; and the
+// list of the slots that were asked to sweep once per launch, which run on the tile list.
+constexpr int kEngLists = 6, kEngPlain = 6, kEngBranches = 7;
+
 struct EngineDev {
     SlotDev *slots;        // max_slots entries
     int max_slots;
     int2 *tiles;           // (slot, tile index within the slot)
     int *ntiles;           // device counter of valid entries in tiles
-    int4 *waves;           // (slot, strip, row block, 0): register-wavefront items of depth-4 slots
-    int *nwaves;           // device counter of valid entries in waves
+    int4 *items;           // register-tile items (slot, first column, first row, last row), by list
+    int *item_off;         // kEngLists + 1 offsets of the lists in items
     SlotStatus *status;    // max_slots entries, refreshed by the advance kernel
 };
 
+// Streams and events of an engine's step: the lists' sweeps are branches of its graph, forked after
+// `decide` and joined before `export`.
+struct EngineBranches {
+    cudaStream_t side[kEngBranches] = {};
+    cudaEvent_t fork = nullptr, join[kEngBranches] = {};
+};
+
 // launchers (engine.cu)
-// one engine step: correct, defect, decide, `sweeps` sweep launches (with wave_grid > 0, each
-// also launches the register-wavefront kernel over the wave list with that many blocks), export,
-// advance (the step's sweeps applied to the counters at once)
-cudaError_t eng_launch_step(const EngineDev &e, int grid_tiles, int grid_slots, size_t sweep_smem,
-                            int sweeps, int wave_grid, cudaStream_t s);
-// Appends the register-wavefront items of a slot (Nx x Ny, stencil st) to items, if the slot's
-// sweeps at depth `depth` run on the wavefront (5- and 9-point slots at depth 4); returns how many.
-int eng_wave_items(int slot, int Nx, int Ny, int st, int depth, std::vector<int4> &items);
-// Blocks of the wavefront kernel resident on the device at once (one wave).
-int eng_wave_grid();
+// one engine step: correct, defect, decide, `sweeps` sweep launches of every list in `lists` (a bit
+// per list; register tiles with rt_blocks blocks), export, advance (the step's sweeps applied at once)
+cudaError_t eng_launch_step(const EngineDev &e, int grid_tiles, int grid_slots, unsigned lists, int rt_blocks,
+                            const EngineBranches &br, int sweeps, cudaStream_t s);
+// The register-tile list of a problem, and its items appended; depth: the slot's sweeps per launch.
+int eng_list(int st, int Nx, int Ny);
+void eng_rt_items(int slot, int Nx, int Ny, int st, int depth, std::vector<int4> &items);
+// The list whose sweep kernel fn is, or -1.
+int eng_list_of_kernel(const void *fn);
+// Sweeps per launch of a problem that does not name them: 8, or 4 of 17 points.
+int eng_default_depth(int st);
 cudaError_t eng_launch_import(const EngineDev &e, int slot, int ntiles, const double *f,
                               long long ldf, const double *u0, long long ldu, cudaStream_t s);
-size_t eng_sweep_smem(int max_depth);
-// blocks of the one-sweep tile kernel (the engine's heaviest in registers) resident per SM
-int eng_sweep_blocks_per_sm();
-// true for the kernels that loop over the tile list (their grid may be any size)
+// true for the kernels that loop over the tile list (their grid may be any size; the sweep among them)
 bool eng_is_tile_kernel(const void *fn);
-cudaError_t eng_prepare(size_t sweep_smem);
+// the sweep kernels' shared-memory limits on the current device
+cudaError_t eng_prepare();

@@ -1,6 +1,5 @@
 // Device arithmetic shared by the kernel translation units: the stencil evaluation in the
-// fixed order of the FP64 reference (y-marching and direct forms), the double-FP64 defect,
-// and the shared-memory stage of the temporal-blocked FP32 sweep.
+// fixed order of the FP64 reference (y-marching and direct forms), and the double-FP64 defect.
 #pragma once
 
 #include "cj_internal.h"
@@ -278,80 +277,6 @@ __device__ __forceinline__ double resid_dd(const double *uh, const double *ul, c
     }
     const double Llo = plain_L<ST>(ul, g, i, j);
     return (s.S + (s.E + D * Llo)) / D;
-}
-
-template <int ST>
-__device__ __forceinline__ float resid_smem(const float *A, int SX, int x, int y, float rk) {
-    auto N = [&](int dx, int dy) { return A[(y + dy) * SX + (x + dx)]; };
-    return resid_diff32<ST>(N, A[y * SX + x], rk);
-}
-
-// One tile of the temporal-blocked FP32 sweep, run by the whole block: `depth` sweeps with
-// weights w[0..depth-1] on the tile whose first interior node is (i0, j0), TX x TY nodes,
-// staged with a halo of r * depth in shared memory `sm` (3 (TX+2H)(TY+2H) floats).  The
-// caller owns the synchronisation before sm is reused.
-template <int ST>
-__device__ __forceinline__ void tb_tile(const float *__restrict__ e, const float *__restrict__ r,
-                                        float *__restrict__ out, const Grid &g, int depth,
-                                        const float *w, int i0, int j0, int TX, int TY, float *sm) {
-    constexpr int R = ST == 17 ? 2 : 1;
-    const int nt = blockDim.x;
-    const int H = R * depth;
-    const int SX = TX + 2 * H, SY = TY + 2 * H, NS = SX * SY;
-    float *A = sm, *B = sm + NS, *Rs = sm + 2 * NS;
-    // node (gx0 + x, gy0 + y) sits at staged cell (x, y)
-    const int gx0 = i0 - H, gy0 = j0 - H;
-    const int Nx = g.Nx, Ny = g.Ny;
-
-    for (int c = threadIdx.x; c < NS; c += nt) {
-        const int x = c % SX, y = c / SX, gi = gx0 + x, gj = gy0 + y;
-        float a = 0.0f, q = 0.0f;
-        if (gi >= -1 && gi <= Nx + 2 && gj >= -1 && gj <= Ny + 2) {
-            const long long k = g.idx(gi, gj);
-            a = __ldg(e + k);
-            q = __ldg(r + k);
-        }
-        A[c] = a;
-        B[c] = a;
-        Rs[c] = q;
-    }
-    __syncthreads();
-
-    for (int s = 1; s <= depth; ++s) {
-        const float ws = w[s - 1];
-        const int lo = R * s, wx = SX - 2 * lo, wy = SY - 2 * lo;
-        for (int c = threadIdx.x; c < wx * wy; c += nt) {
-            const int x = lo + c % wx, y = lo + c / wx, gi = gx0 + x, gj = gy0 + y;
-            if (gi >= 1 && gi <= Nx && gj >= 1 && gj <= Ny) {
-                const float uc = A[y * SX + x];
-                B[y * SX + x] = fmaf(ws, resid_smem<ST>(A, SX, x, y, Rs[y * SX + x]), uc);
-            }
-        }
-        __syncthreads();
-        if (R == 2) {
-            // outer ghost layer of the new values: odd reflection of the interior
-            for (int c = threadIdx.x; c < wx * wy; c += nt) {
-                const int x = lo + c % wx, y = lo + c / wx, gi = gx0 + x, gj = gy0 + y;
-                const bool gx = gi == -1 || gi == Nx + 2, gy = gj == -1 || gj == Ny + 2;
-                if (!(gx || gy)) continue;
-                if (gi < -1 || gi > Nx + 2 || gj < -1 || gj > Ny + 2) continue;
-                if (gi == 0 || gi == Nx + 1 || gj == 0 || gj == Ny + 1) continue;
-                const int mx = gi == -1 ? x + 2 : gi == Nx + 2 ? x - 2 : x;
-                const int my = gj == -1 ? y + 2 : gj == Ny + 2 ? y - 2 : y;
-                const float v = B[my * SX + mx];
-                B[y * SX + x] = (gx != gy) ? -v : v;
-            }
-            __syncthreads();
-        }
-        float *t = A;
-        A = B;
-        B = t;
-    }
-
-    for (int c = threadIdx.x; c < TX * TY; c += nt) {
-        const int x = H + c % TX, y = H + c / TX, gi = gx0 + x, gj = gy0 + y;
-        if (gi <= Nx && gj <= Ny) store_node<R, float>(out, g, gi, gj, A[y * SX + x]);
-    }
 }
 
 }  // namespace
