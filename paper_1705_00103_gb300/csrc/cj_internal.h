@@ -39,6 +39,12 @@ struct March {
     int blocks() const { return nbx * nby; }
 };
 
+// Launch shape of the FP64 sweep (sweep64.cu): threads 0 .. Nx chunks - 1, one column each of a chunk
+// of ty rows.
+struct Sweep64Shape {
+    int ty, chunks, blocks;
+};
+
 struct cj_plan {
     int Nx, Ny, st, r, precision, literal_n, bc;
     int method = 0;           // cj_method: CJ_CJM or CJ_JACOBI (every w_n = 1/c)
@@ -51,6 +57,7 @@ struct cj_plan {
     int device;
     Grid g64, g32;
     March m64, m32;
+    Sweep64Shape s64{};
     double *u0 = nullptr, *u1 = nullptr, *b = nullptr;    // padded FP64
     float *e0 = nullptr, *e1 = nullptr, *rt = nullptr;    // padded FP32 (mixed only)
     double *d0 = nullptr, *d1 = nullptr, *r64 = nullptr;  // padded FP64 correction ping-pong and
@@ -133,6 +140,17 @@ int cluster_solve_size(const cj_plan *p);
 // res_dev[0..5] = status, sweeps, cycles, rho, rinf, fl
 cudaError_t launch_cluster_solve(const cj_plan *p, double *res_dev, cudaStream_t s);
 
+// ---- the FP64 sweep (sweep64.cu); its launches may overlap the end of the one before in the stream
+Sweep64Shape sweep64_shape(int Nx, int Ny, int st);
+cudaError_t launch_sweep64(const cj_plan *p, const double *u, double *out, double w,
+                           cudaStream_t s);
+// the same with weight w_dev[*pos + k] (graph.cu)
+cudaError_t launch_sweep64_tab(const cj_plan *p, const double *u, double *out, int k, cudaStream_t s);
+// FP64 sweep of the error equation L e = rhs with the homogeneous boundary of the plan's stencil
+// (odd reflection for 17 points whatever the plan's bc): the inner cycle of CJ_FP64_INNER_DD
+cudaError_t launch_sweep64_err(const cj_plan *p, const double *e, const double *rhs, double *out,
+                               double w, cudaStream_t s);
+
 // ---- kernel launchers (kernels.cu); every launcher returns the launch error
 March plan_march(int Nx, int Ny, int st, bool fp64);
 // caller grids -> padded b = h^2 f and u; red[3..4] = (sum b^2, max |b|)
@@ -145,12 +163,6 @@ cudaError_t launch_real_error(const cj_plan *p, const double *u_pad, const doubl
                               cudaStream_t s);
 cudaError_t launch_export(const cj_plan *p, const double *u_pad, double *u, long long ldu,
                           cudaStream_t s);
-cudaError_t launch_sweep64(const cj_plan *p, const double *u, double *out, double w,
-                           cudaStream_t s);
-// FP64 sweep of the error equation L e = rhs with the homogeneous boundary of the plan's stencil
-// (odd reflection for 17 points whatever the plan's bc): the inner cycle of CJ_FP64_INNER_DD
-cudaError_t launch_sweep64_err(const cj_plan *p, const double *e, const double *rhs, double *out,
-                               double w, cudaStream_t s);
 cudaError_t launch_sweep32(const cj_plan *p, const float *e, const float *r, float *out, float w,
                            cudaStream_t s);
 // residual of u_pad against p->b: red[0..2] = (sum r^2, max|r|, sum u^2); with rt != NULL

@@ -1,11 +1,10 @@
 // Device kernels of the Chebyshev-Jacobi solver for sm_103a.
 //
-// Hot kernel: the weighted sweep u' = u + w_n (L u - b) of Sec. 2.1 for the 5-point
-// (Table 3), 9-point (Eq. 1) and 17-point (Eq. 2) Laplacians.  A stencil is not a dense
-// contraction, so there are no tensor cores here.  On GB300 the FP64 pipe issues about
-// two FMAs per SM clock (~0.6 T instructions/s; FP32 issues ~60x more), so the FP64 sweep
-// is bound by FP64 instruction issue, not by HBM: the kernels below evaluate L u - b in
-// the fewest FP64 instructions, and every FP64 addition is issued as fma(a, one, b)
+// The imports, exports, residuals and corrections around the sweeps (the FP64 sweep itself is
+// sweep64.cu's).  A stencil is not a dense contraction, so there are no tensor cores here.  On
+// GB300 the FP64 pipe issues about two FMAs per SM clock (~0.6 T instructions/s; FP32 issues ~60x
+// more), so FP64 stencil evaluation is bound by FP64 instruction issue, not by HBM: L u - b is
+// evaluated in the fewest FP64 instructions, and every FP64 addition is issued as fma(a, one, b)
 // (bit-identical to a + b; the FMA path has the higher issue rate on this part).
 //
 // Evaluation order of L u - b (fixed, shared by design with the FP64 reference):
@@ -27,35 +26,6 @@
 #include "stencil_dev.cuh"
 
 namespace {
-
-// Stores the updated node; for the 17-point stencil with MIRROR also its reflection ghosts
-// (without MIRROR the ghost ring holds fixed Dirichlet data).
-template <int ST, typename T, bool MIRROR = true>
-struct SweepOp {
-    T *out;
-    const Grid *g;
-    int i;
-    T w;
-    __device__ __forceinline__ void operator()(int j, T r, T uc) {
-        store_node<((ST == 17 && MIRROR) ? 2 : 1)>(out, *g, i, j, Ar<T>::fm(w, r, uc));
-    }
-};
-
-// One FP64 weighted sweep: out = u + w (L u - b) in the pair-sum order above (the FP32 inner
-// sweep, in difference form, is sweep32.cu's).
-// MIRROR: rewrite the odd-reflection ghosts of the 17-point stencil (homogeneous boundary);
-// without it the ghost ring holds fixed Dirichlet data and is left alone.
-template <int ST, typename T, bool MIRROR = true>
-__global__ void __launch_bounds__(kBX) sweep_kernel(const T *__restrict__ u,
-                                                    const T *__restrict__ b, T *__restrict__ out,
-                                                    Grid g, int ty, T w, T one) {
-    const int i = blockIdx.x * kBX + threadIdx.x + 1;
-    const int j0 = blockIdx.y * ty + 1;
-    const int j1 = min(j0 + ty - 1, g.Ny);
-    if (i > g.Nx) return;
-    SweepOp<ST, T, MIRROR> op{out, &g, i, w};
-    march<ST, T>(u, b, g, i, j0, j1, one, op);
-}
 
 struct ResidOp {
     double s2 = 0.0, mx = 0.0, u2 = 0.0;
@@ -239,33 +209,6 @@ March plan_march(int Nx, int Ny, int st, bool fp64) {
     m.nby = (Ny + m.ty - 1) / m.ty;
     (void)st;
     return m;
-}
-
-cudaError_t launch_sweep64(const cj_plan *p, const double *u, double *out, double w,
-                           cudaStream_t s) {
-    dim3 grid(p->m64.nbx, p->m64.nby);
-    switch (p->st) {
-        case 5: sweep_kernel<5, double><<<grid, kBX, 0, s>>>(u, p->b, out, p->g64, p->m64.ty, w, 1.0); break;
-        case 9: sweep_kernel<9, double><<<grid, kBX, 0, s>>>(u, p->b, out, p->g64, p->m64.ty, w, 1.0); break;
-        default:
-            if (p->bc == CJ_BC_DIRICHLET)
-                sweep_kernel<17, double, false><<<grid, kBX, 0, s>>>(u, p->b, out, p->g64, p->m64.ty, w, 1.0);
-            else
-                sweep_kernel<17, double><<<grid, kBX, 0, s>>>(u, p->b, out, p->g64, p->m64.ty, w, 1.0);
-            break;
-    }
-    return cudaGetLastError();
-}
-
-cudaError_t launch_sweep64_err(const cj_plan *p, const double *e, const double *rhs, double *out,
-                               double w, cudaStream_t s) {
-    dim3 grid(p->m64.nbx, p->m64.nby);
-    switch (p->st) {
-        case 5: sweep_kernel<5, double><<<grid, kBX, 0, s>>>(e, rhs, out, p->g64, p->m64.ty, w, 1.0); break;
-        case 9: sweep_kernel<9, double><<<grid, kBX, 0, s>>>(e, rhs, out, p->g64, p->m64.ty, w, 1.0); break;
-        default: sweep_kernel<17, double><<<grid, kBX, 0, s>>>(e, rhs, out, p->g64, p->m64.ty, w, 1.0); break;
-    }
-    return cudaGetLastError();
 }
 
 // Dirichlet data g (node (i, j) at g[(j+1) ldg + i+1], i, j in -1..N+2) into the ghost ring of

@@ -697,6 +697,7 @@ cj_status cj_plan_create(int Nx, int Ny, cj_stencil st, cj_bc bc, double tol,
     p->g32 = make_grid(Nx, Ny, 4);
     p->m64 = plan_march(Nx, Ny, st, true);
     p->m32 = plan_march(Nx, Ny, st, false);
+    p->s64 = sweep64_shape(Nx, Ny, st);
     long long copy_parts = (long long)((Nx + kBX - 1) / kBX) * (Ny < 1024 ? Ny : 1024);
     long long parts = p->m64.blocks();
     if (copy_parts > parts) parts = copy_parts;
