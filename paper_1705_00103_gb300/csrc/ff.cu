@@ -6,259 +6,336 @@
 // with |lo| <= ulp(hi)/2 (48 significant bits against FP64's 53), and the sweep
 // u' = u + w (L u - b) of Sec. 2.1 is evaluated with the error-free transformations of Knuth
 // (TwoSum: s + e = a + b exactly) and Dekker (TwoProduct, here in its fused-multiply-add form:
-// p + e = a b exactly).  17 points: in the evaluation order of the FP64 sweep (the shared y-march
-// of stencil_dev.cuh, with float-float in place of double).  5 and 9 points: a y-march of its own,
-// with the next row's loads issued ahead, in the algebraically equal scaled form
+// p + e = a b exactly).  17 points: in the evaluation order of the FP64 sweep.  5 and 9 points: in
+// the algebraically equal scaled form
 //   u' = (1 - c w / D) u + (w / D) (S - D b),
 // S the neighbour sum of D L u + c u with coefficients 1 and 4 (D = 1, c = 4 for 5 points; D = 6,
 // c = 20 for 9 points, Eq. 1 times 6): S needs float-float adds and one exact scaling by 4, D b is
-// formed once when b is converted, and w / D and 1 - c w / D are rounded once per sweep on the host
-// -- 69 and 93 FP32 operations per update against 80 and 116 for the three float-float
+// formed once on import, and w / D and 1 - c w / D are rounded once per sweep on the host
+// -- 69 and 91 FP32 operations per update against 80 and 116 for the three float-float
 // multiply-adds of the FP64 sweep's form.  The pair occupies the same 8 bytes as a double,
 // so the sweep moves the FP64 sweep's bytes with FP32 instructions only.  The result is not the
 // FP64 sweep's bits: it agrees with it to a few units of 2^-47 of the terms it adds (in the scaled
 // form, |c1 u| and |w / D| |S - D b|, each at most about 3.4 |w| max|u| + |w| max|b| for 9 points), well
 // inside the per-sweep tolerance of 1e-12 x (max|u| + |w| (9 max|u| + max|b|)) the sweeps are held to.
 //
-// Conversions: the plan's padded FP64 buffers are converted in place to float-float before the
-// sweeps (hi = fl32(d), lo = fl32(d - hi)) and back after them (fl64(hi + lo)); values must lie in
-// the float range (|d| < 3.4e38); below 2^-126 their low part is lost (relative error 2^-24 of a
-// value that small).  Homogeneous-Dirichlet plans only: their ghost ring is 0 or the reflection of
-// the interior, which the sweeps rewrite, so no boundary data passes through the conversions.
+// What bounds it: HBM (24 bytes a node) for 5 and 9 points, FP32 issue for 17 (about 190 operations
+// a node).  A thread
+// holds two adjacent columns as pairs (hi, hi) and (lo, lo), so that every operation is one packed
+// instruction for both, and walks ty rows with the next row's loads one iteration ahead.  In memory
+// a pair of columns is (hi, hi, lo, lo), 16 bytes: one load brings both operands of the packed
+// instructions to their registers.  The import writes this form straight from the caller's arrays
+// and the export reads it, so no conversion passes stand between them and the sweeps.  Values must
+// lie in the float range (|d| < 3.4e38); below 2^-126 their low part is lost (relative error 2^-24
+// of a value that small).  Homogeneous-Dirichlet plans only: their ghost ring is 0 or the
+// reflection of the interior, which the sweeps rewrite.
+//
+// Measured on one GB300, 4095 x 4001 (one column a thread with scalar operations and conversion
+// passes -> this): 9 points 83.7 -> 67.0 us a sweep (245 Gupd/s, 0.88 of the copy bandwidth), 5
+// points 68.2 -> 64.0, 17 points 167 -> 121; import and export 1190 -> 177 us; 9-point 333 x 250:
+// 5.7 -> 2.3 us a sweep.
 #include "cj_internal.h"
-#include "grid_dev.cuh"
-#include "stencil_dev.cuh"
 
 namespace {
 
-struct __align__(8) ff {
+struct ff {
     float hi, lo;
 };
 
-__device__ __forceinline__ ff operator-(ff a) { return ff{-a.hi, -a.lo}; }
-
-// Knuth's TwoSum: s + e = a + b exactly (6 operations, no condition on |a|, |b|).
-__device__ __forceinline__ ff two_sum_f(float a, float b) {
-    const float s = a + b;
-    const float bb = s - a;
-    const float e = (a - (s - bb)) + (b - bb);
-    return ff{s, e};
-}
-
-// Dekker's FastTwoSum: s + e = a + b exactly when |a| >= |b| (or a = 0).
-__device__ __forceinline__ ff fast_two_sum_f(float a, float b) {
-    const float s = a + b;
-    return ff{s, b - (s - a)};
-}
-
-// a + b: TwoSum of the high parts, the low parts added to its error, renormalised; the error is a
-// few units of 2^-47 of |a| + |b|.
-__device__ __forceinline__ ff ff_add(ff a, ff b) {
-    const ff s = two_sum_f(a.hi, b.hi);
-    return fast_two_sum_f(s.hi, s.lo + (a.lo + b.lo));
-}
-
-// a * b: the exact product of the high parts by a fused multiply-add (TwoProduct), the cross
-// terms added to its error, renormalised.
-__device__ __forceinline__ ff ff_mul(ff a, ff b) {
-    const float p = a.hi * b.hi;
-    float e = fmaf(a.hi, b.hi, -p);
-    e = fmaf(a.hi, b.lo, e);
-    e = fmaf(a.lo, b.hi, e);
-    return fast_two_sum_f(p, e);
-}
-
-// a - b
-__device__ __forceinline__ ff ff_sub(ff a, ff b) { return ff_add(a, -b); }
-
-// a times a power of two (exact: both parts scale without rounding)
-__device__ __forceinline__ ff ff_scale2(ff a, float two_k) { return ff{a.hi * two_k, a.lo * two_k}; }
-
-// float-float of a double, rounded once per part (host and device)
+// float-float of a double, rounded once per part
 __host__ __device__ __forceinline__ ff ff_of(double d) {
     const float hi = (float)d;
     return ff{hi, (float)(d - (double)hi)};
 }
 
-}  // namespace
+// The same on the integer pipe (a conversion between the types occupies the FP64 pipe like an
+// operation, and ff_of takes four): the mantissa rounded to 24 bits, ties to even, and the remainder,
+// below 2^29, as an integer.  Zeros, and values whose parts leave the normal float range, go the other way.
+__device__ __forceinline__ ff ff_of_bits(double d) {
+    const unsigned hw = (unsigned)__double2hiint(d), lw = (unsigned)__double2loint(d);
+    const int e = (int)(hw >> 20 & 0x7ffu) - 1023;
+    if ((unsigned)(e + 73) > 199u)  // not 2^-73 <= |d| < 2^127
+        return (hw << 1 | lw) == 0 ? ff{__uint_as_float(hw), 0.0f} : ff_of(d);
+    const unsigned m = __funnelshift_l(lw, hw & 0xfffffu | 0x100000u, 3);  // leading 24 bits
+    const unsigned rest = lw & 0x1fffffffu;
+    const unsigned up = (rest + 0x0fffffffu + (m & 1u)) >> 29;
+    const int rem = (int)rest - (int)(up << 29);
+    const unsigned sign = hw & 0x80000000u;
+    const float hi = __uint_as_float(sign | (((unsigned)(e + 126) << 23) + m + up));
+    const float unit = __uint_as_float(sign | ((unsigned)(e + 75) << 23));  // 2^(e - 52), signed
+    return ff{hi, (float)rem * unit};
+}
 
-namespace {
+// fl64 of a float, on the integer pipe where it is normal or 0
+__device__ __forceinline__ double double_of(float x) {
+    const unsigned b = __float_as_uint(x), e = b >> 23 & 0xffu;
+    if (e - 1u > 253u) return (b << 1) == 0 ? __hiloint2double((int)b, 0) : (double)x;
+    return __hiloint2double((int)((b & 0x80000000u) | ((b & 0x7fffffffu) >> 3) + (896u << 20)), (int)(b << 29));
+}
 
-template <>
-struct Ar<ff> {
-    static __device__ __forceinline__ ff add(ff a, ff b, ff) { return ff_add(a, b); }
-    static __device__ __forceinline__ ff fm(ff a, ff b, ff c) { return ff_add(ff_mul(a, b), c); }
+// ---- two columns' values, packed: each half rounded like the scalar instruction
+
+__device__ __forceinline__ float2 bc(float c) { return make_float2(c, c); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, bc(-1.0f), a); }
+
+struct ff2 {
+    float2 h, l;
 };
 
-// The stencil coefficients of h^2 Delta_h as float-float (each rounded once from its FP64 value).
-template <>
-struct Co<ff> {
-    static __device__ __forceinline__ ff c5() { return ff{-4.0f, 0.0f}; }
-    static __device__ __forceinline__ ff ax9() { return ff_of(4.0 / 6.0); }
-    static __device__ __forceinline__ ff dg9() { return ff_of(1.0 / 6.0); }
-    static __device__ __forceinline__ ff cc9() { return ff_of(-20.0 / 6.0); }
-    static __device__ __forceinline__ ff a1() { return ff_of(64.0 / 72.0); }
-    static __device__ __forceinline__ ff a2() { return ff_of(-4.0 / 72.0); }
-    static __device__ __forceinline__ ff d1() { return ff_of(16.0 / 72.0); }
-    static __device__ __forceinline__ ff d2() { return ff_of(-1.0 / 72.0); }
-    static __device__ __forceinline__ ff cc17() { return ff_of(-300.0 / 72.0); }
-};
+__device__ __forceinline__ ff2 ff2_of(const float4 &q) { return ff2{make_float2(q.x, q.y), make_float2(q.z, q.w)}; }
 
-template <>
-__device__ __forceinline__ ff ld<ff>(const ff *p) {
-    const float2 v = __ldg(reinterpret_cast<const float2 *>(p));
-    return ff{v.x, v.y};
+// Dekker's FastTwoSum: s + e = a + b exactly when |a| >= |b| (or a = 0).
+__device__ __forceinline__ ff2 fast_two_sum(float2 a, float2 b) {
+    const float2 s = add2(a, b);
+    return ff2{s, sub2(b, sub2(s, a))};
+}
+
+// a + b: Knuth's TwoSum of the high parts (6 operations, no condition on |a|, |b|), the low parts
+// added to its error, renormalised; the error is a few units of 2^-47 of |a| + |b|.
+__device__ __forceinline__ ff2 ff_add(const ff2 &a, const ff2 &b) {
+    const float2 s = add2(a.h, b.h), bb = sub2(s, a.h);
+    const float2 e = add2(sub2(a.h, sub2(s, bb)), sub2(b.h, bb));
+    return fast_two_sum(s, add2(e, add2(a.l, b.l)));
+}
+
+// 4 a + b: the same with 4 a, which is exact, inside the operations that read a
+__device__ __forceinline__ ff2 ff_add4(const ff2 &a, const ff2 &b) {
+    const float2 four = bc(4.0f);
+    const float2 s = fma2(a.h, four, b.h), bb = fma2(a.h, bc(-4.0f), s);
+    const float2 e = add2(fma2(a.h, four, sub2(bb, s)), sub2(b.h, bb));
+    return fast_two_sum(s, add2(e, fma2(a.l, four, b.l)));
+}
+
+// c a for a constant c: the exact product of the high parts by a fused multiply-add (TwoProduct),
+// formed negated for it, the cross terms added to its error, renormalised.
+__device__ __forceinline__ ff2 ff_mul(ff c, const ff2 &a) {
+    const float2 np = __fmul2_rn(bc(-c.hi), a.h);
+    float2 e = fma2(bc(c.hi), a.h, np);
+    e = fma2(bc(c.hi), a.l, e);
+    e = fma2(bc(c.lo), a.h, e);
+    const float2 s = sub2(e, np);
+    return ff2{s, sub2(e, add2(s, np))};
+}
+
+// c a + b
+__device__ __forceinline__ ff2 ff_fma(ff c, const ff2 &a, const ff2 &b) { return ff_add(ff_mul(c, a), b); }
+
+// ---- the packed grid: node k of the padded layout has its high part at float 4 (k / 2) + k % 2 and
+// its low part two floats on; columns c, c + 1 with odd c share 16 bytes
+
+__host__ __device__ __forceinline__ long long ff_pos(long long k) { return ((k >> 1) << 2) + (k & 1); }
+
+__device__ __forceinline__ void ff_put(float *a, long long k, ff v) {
+    a[ff_pos(k)] = v.hi;
+    a[ff_pos(k) + 2] = v.lo;
+}
+
+// Writes v at interior node (i, j) and, for the 17-point stencil, the reflections that mirror it.
+template <int R>
+__device__ __forceinline__ void ff_store(float *a, const Grid &g, int i, int j, ff v) {
+    ff_put(a, g.idx(i, j), v);
+    if (R == 2) {
+        const ff nv{-v.hi, -v.lo};
+        const bool x0 = i == 1, x1 = i == g.Nx;
+        if (x0) ff_put(a, g.idx(-1, j), nv);
+        if (x1) ff_put(a, g.idx(g.Nx + 2, j), nv);
+        if (j == 1) {
+            ff_put(a, g.idx(i, -1), nv);
+            if (x0) ff_put(a, g.idx(-1, -1), v);
+            if (x1) ff_put(a, g.idx(g.Nx + 2, -1), v);
+        }
+        if (j == g.Ny) {
+            ff_put(a, g.idx(i, g.Ny + 2), nv);
+            if (x0) ff_put(a, g.idx(-1, g.Ny + 2), v);
+            if (x1) ff_put(a, g.idx(g.Nx + 2, g.Ny + 2), v);
+        }
+    }
 }
 
 // The weights of one sweep.  17 points: w, for u' = u + w (L u - b) in the FP64 sweep's order.
 // 5 and 9 points, in the scaled form D L u = sum of the neighbours with small integer
-// coefficients - c u (D = 1, c = 4; D = 6, c = 20), with b stored as D b:
+// coefficients - c u (D = 1, c = 4; D = 6, c = 20), with b stored as -D b:
 //   u' = c1 u + wD (D L u + c u - D b),   wD = w / D,   c1 = 1 - c wD,
 // so the neighbour sum needs no multiplication (its coefficients 1 and 4 are powers of two).
-struct FFWeights {
+struct FFArgs {
+    const float *u, *nb;
+    float *out;
+    Grid g;
+    int ty, chunks;
     ff w, wD, c1;
 };
 
-template <int ST>
-struct SweepOpFF {
-    ff *out;
-    const Grid *g;
-    int i;
-    FFWeights w;
-    __device__ __forceinline__ void operator()(int j, ff r, ff uc) {
-        store_node<(ST == 17 ? 2 : 1), ff>(out, *g, i, j, Ar<ff>::fm(w.w, r, uc));
-    }
-    // t = D L u + c u - D b at (i, j): the new value c1 u + wD t
-    __device__ __forceinline__ void scaled(int j, ff t, ff uc) {
-        store_node<1, ff>(out, *g, i, j, ff_add(ff_mul(w.c1, uc), ff_mul(w.wD, t)));
-    }
+constexpr int kFFThreads = 128;
+
+// One row of a thread's pair of columns: the pair, and the pairs to its left and right.
+struct FFRow {
+    float4 l, c, r;
 };
 
-// Blocks of kBX threads resident per SM: 16 (32 registers a thread) for the 5- and 9-point
-// sweeps, 10 for the 17-point one, whose five-row window needs about 50.
-__host__ __device__ constexpr int ff_blocks_per_sm(int st) { return st == 17 ? 10 : 16; }
+__device__ __forceinline__ FFRow ff_row(const float4 *p) { return FFRow{__ldca(p - 1), __ldca(p), __ldca(p + 1)}; }
 
-// The y-march of the 5- and 9-point sweeps (the FP64 sweep's order), with the loads of row j + 1
-// (and b of row j) issued one iteration ahead: each iteration's dependent float-float chain is
-// long, so the next row's memory latency is hidden behind it.  Row indices are clamped to the
-// strip's last row + 1 (a row every strip has), so the last iteration reloads it harmlessly.
+// u(i-1) + u(i+1) and u(i-2) + u(i+2) of both columns
+__device__ __forceinline__ ff2 ff_side1(const FFRow &q) {
+    return ff_add(ff2{make_float2(q.l.y, q.c.x), make_float2(q.l.w, q.c.z)},
+                  ff2{make_float2(q.c.y, q.r.x), make_float2(q.c.w, q.r.z)});
+}
+__device__ __forceinline__ ff2 ff_side2(const FFRow &q) { return ff_add(ff2_of(q.l), ff2_of(q.r)); }
+
+// One weighted sweep out = u + w (L u - b): thread t has pair t mod np of chunk t / np, rows
+// chunk ty + 1 onwards.  Its launches overlap the end of the one before: nothing is read before
+// griddepcontrol.wait, which makes that sweep's stores visible.
 template <int ST>
-__device__ __forceinline__ void march_ff(const ff *__restrict__ u, const ff *__restrict__ b, const Grid &g,
-                                         int i, int j0, int j1, SweepOpFF<ST> &op) {
-    const long long P = g.pitch;
-    const ff *col = u + g.idx(i, 0);
-    const ff *bcol = b + g.idx(i, 0);
-    if (ST == 5) {
-        ff um = ld(col + (long long)(j0 - 1) * P);
-        ff uc = ld(col + (long long)j0 * P);
-        const ff *row = col + (long long)j0 * P;
-        ff nu = ld(row + P), nl = ld(row - 1), nr = ld(row + 1), nb = ld(bcol + (long long)j0 * P);
+__global__ void __launch_bounds__(kFFThreads, ST == 17 ? 4 : 7) sweep_ff_kernel(const __grid_constant__ FFArgs a) {
+    constexpr int R = ST == 17 ? 2 : 1;
+    const Grid &g = a.g;
+    const int np = (g.Nx + 1) / 2;
+    const int t = (int)(blockIdx.x * kFFThreads + threadIdx.x);
+    const int ch = t / np, i = 2 * (t - ch * np) + 1;
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+    if (ch >= a.chunks) return;
+    const int j0 = ch * a.ty + 1, j1 = min(j0 + a.ty - 1, g.Ny);
+    const long long P = g.pitch / 2;  // pairs per row
+    const bool both = i < g.Nx;
+    const float4 *row = reinterpret_cast<const float4 *>(a.u) + g.idx(i, j0 - R) / 2;
+    const float4 *bp = reinterpret_cast<const float4 *>(a.nb) + g.idx(i, j0) / 2;
+    float4 *op = reinterpret_cast<float4 *>(a.out) + g.idx(i, j0) / 2;
+    auto store = [&](int j, const ff2 &v) {
+        const bool edge = R == 2 && (i == 1 || i + 1 >= g.Nx || j == 1 || j == g.Ny);
+        if (both && !edge) {
+            *op = make_float4(v.h.x, v.h.y, v.l.x, v.l.y);
+        } else {
+            ff_store<R>(a.out, g, i, j, ff{v.h.x, v.l.x});
+            if (both) ff_store<R>(a.out, g, i + 1, j, ff{v.h.y, v.l.y});
+        }
+        op += P;
+    };
+    if constexpr (ST != 17) {
+        ff2 um = ff2_of(__ldca(row)), pm, pc;
+        if (ST == 9) pm = ff_side1(ff_row(row));
+        row += P;
+        FFRow c = ff_row(row);  // 5 points: row j; 9 points: of row j only the pair is used in the loop
+        ff2 uc = ff2_of(c.c);
+        if (ST == 9) {
+            pc = ff_side1(c);
+            row += P;
+        }
+        // 5 points: row j's sides and row j + 1's pair; 9 points: row j + 1
+        FFRow n = ST == 9 ? ff_row(row) : FFRow{c.l, __ldca(row + P), c.r};
+        float4 nb = __ldcs(bp);
+#pragma unroll 2
         for (int j = j0; j <= j1; ++j) {
-            const ff up = nu, l = nl, r_ = nr, bk = nb;
-            const int jn = min(j + 1, j1);
-            row = col + (long long)jn * P;
-            nu = ld(row + P);
-            nl = ld(row - 1);
-            nr = ld(row + 1);
-            nb = ld(bcol + (long long)jn * P);
-            const ff p0 = ff_add(l, r_);
-            const ff v1 = ff_add(um, up);
-            const ff a = ff_add(p0, v1);
-            op.scaled(j, ff_sub(a, bk), uc);
+            const FFRow q = n;
+            const ff2 bk = ff2_of(nb), up = ff2_of(q.c);
+            const long long step = j < j1 ? P : 0;  // the last row loads itself again
+            row += step;
+            bp += step;
+            n = ff_row(row);
+            if (ST == 5) n.c = __ldca(row + P);
+            nb = __ldcs(bp);
+            ff2 s;
+            if (ST == 5) {
+                const FFRow e{q.l, make_float4(uc.h.x, uc.h.y, uc.l.x, uc.l.y), q.r};
+                s = ff_add(ff_side1(e), ff_add(um, up));
+            } else {
+                const ff2 pp = ff_side1(q);
+                s = ff_add4(ff_add(pc, ff_add(um, up)), ff_add(pm, pp));
+                pm = pc;
+                pc = pp;
+            }
+            store(j, ff_add(ff_mul(a.c1, uc), ff_mul(a.wD, ff_add(s, bk))));
             um = uc;
             uc = up;
         }
     } else {
-        const ff *row = col + (long long)(j0 - 1) * P;
-        ff um = ld(row);
-        ff pm = ff_add(ld(row - 1), ld(row + 1));
-        row += P;
-        ff uc = ld(row);
-        ff pc = ff_add(ld(row - 1), ld(row + 1));
-        row += P;
-        ff nu = ld(row), nl = ld(row - 1), nr = ld(row + 1), nb = ld(bcol + (long long)j0 * P);
-        // unrolled by 2, so the rotation of the window (um, uc, pm, pc and the rows in flight)
-        // is register renaming rather than moves: 160 -> 170 Gupd/s on 4096^2
-#pragma unroll 2
+        // rows j-2 .. j+1 in registers on entry to each iteration: the pair and its side sums
+        ff2 u_[4], p_[4], Q_[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const FFRow q = ff_row(row);
+            u_[k] = ff2_of(q.c);
+            p_[k] = ff_side1(q);
+            Q_[k] = ff_side2(q);
+            row += P;
+        }
+        FFRow n = ff_row(row);
+        float4 nb = __ldcs(bp);
+#pragma unroll 1
         for (int j = j0; j <= j1; ++j) {
-            const ff up = nu, l = nl, r_ = nr, bk = nb;
-            const int jn = min(j + 1, j1);
-            row = col + (long long)(jn + 1) * P;
-            nu = ld(row);
-            nl = ld(row - 1);
-            nr = ld(row + 1);
-            nb = ld(bcol + (long long)jn * P);
-            const ff pp = ff_add(l, r_);
-            const ff v1 = ff_add(um, up);
-            const ff a = ff_add(pc, v1);
-            const ff d = ff_add(pm, pp);
-            op.scaled(j, ff_sub(ff_add(ff_scale2(a, 4.0f), d), bk), uc);
-            um = uc;
-            uc = up;
-            pm = pc;
-            pc = pp;
+            const FFRow q = n;
+            const ff2 bk = ff2_of(nb), u4 = ff2_of(q.c);
+            const long long step = j < j1 ? P : 0;
+            row += step;
+            bp += step;
+            n = ff_row(row);
+            nb = __ldcs(bp);
+            const ff2 p4 = ff_side1(q), Q4 = ff_side2(q);
+            const ff2 a1 = ff_add(p_[2], ff_add(u_[1], u_[3])), a2 = ff_add(Q_[2], ff_add(u_[0], u4));
+            const ff2 d1 = ff_add(p_[1], p_[3]), d2 = ff_add(Q_[0], Q4);
+            const ff2 r = ff_fma(
+                ff_of(64.0 / 72.0), a1,
+                ff_fma(ff_of(-4.0 / 72.0), a2,
+                       ff_fma(ff_of(16.0 / 72.0), d1,
+                              ff_fma(ff_of(-1.0 / 72.0), d2, ff_fma(ff_of(-300.0 / 72.0), u_[2], bk)))));
+            store(j, ff_fma(a.w, r, u_[2]));
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                u_[k] = u_[k + 1];
+                p_[k] = p_[k + 1];
+                Q_[k] = Q_[k + 1];
+            }
+            u_[3] = u4;
+            p_[3] = p4;
+            Q_[3] = Q4;
         }
     }
 }
 
-// One weighted sweep out = u + w (L u - b) in float-float on the padded grids (homogeneous plans:
-// the 17-point stencil's reflection ghosts are rewritten with each node).
-template <int ST>
-__global__ void __launch_bounds__(kBX, ff_blocks_per_sm(ST)) sweep_ff_kernel(const ff *__restrict__ u,
-                                                                        const ff *__restrict__ b,
-                                                                        ff *__restrict__ out, Grid g, int ty,
-                                                                        FFWeights w) {
+// Caller grids -> packed u and nb = -D h^2 f.
+template <int R>
+__global__ void __launch_bounds__(kBX) import_ff_kernel(const double *__restrict__ f, long long ldf,
+                                                        const double *__restrict__ uin, long long ldu, float *nb,
+                                                        float *u, Grid g, double h2, double D) {
     const int i = blockIdx.x * kBX + threadIdx.x + 1;
-    const int j0 = blockIdx.y * ty + 1;
-    const int j1 = min(j0 + ty - 1, g.Ny);
     if (i > g.Nx) return;
-    SweepOpFF<ST> op{out, &g, i, w};
-    if (ST == 17)
-        march<ST, ff>(u, b, g, i, j0, j1, ff{1.0f, 0.0f}, op);
-    else
-        march_ff<ST>(u, b, g, i, j0, j1, op);
-}
-
-// Launch shape: 128-column strips of ty rows, about ff_blocks_per_sm blocks per SM in one wave
-// (rows per strip at least 4, 8 for the 17-point stencil, against the rows a strip re-reads).
-dim3 ff_grid(const Grid &g, int st, int *ty) {
-    const int nbx = (g.Nx + kBX - 1) / kBX;
-    int sms = 0, dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    long long nby = (long long)(sms > 0 ? sms : 1) * ff_blocks_per_sm(st) / nbx;
-    if (nby < 1) nby = 1;
-    if (nby > g.Ny) nby = g.Ny;
-    const int min_ty = st == 17 ? 8 : 4;
-    int t = (int)((g.Ny + nby - 1) / nby);
-    if (t < min_ty) t = min_ty < g.Ny ? min_ty : g.Ny;
-    *ty = t;
-    return dim3(nbx, (g.Ny + t - 1) / t);
-}
-
-// In place: doubles -> float-float pairs of D times them (D = 1 for u; the scale of the sweep's
-// form for b), and back (times 1 / D, exact for D = 1; b is imported again by every call that
-// uses it, so its value after the sweeps is not read).
-__global__ void __launch_bounds__(256) to_ff_kernel(double *a, long long n, double D) {
-    for (long long k = blockIdx.x * 256LL + threadIdx.x; k < n; k += (long long)gridDim.x * 256) {
-        const ff v = ff_of(D * a[k]);
-        reinterpret_cast<ff *>(a)[k] = v;
+    for (int j = blockIdx.y + 1; j <= g.Ny; j += gridDim.y) {
+        const double bk = h2 * f[(long long)(j - 1) * ldf + (i - 1)];
+        ff_put(nb, g.idx(i, j), ff_of_bits(-(D * bk)));
+        ff_store<R>(u, g, i, j, ff_of_bits(uin[(long long)(j - 1) * ldu + (i - 1)]));
     }
 }
 
-__global__ void __launch_bounds__(256) from_ff_kernel(double *a, long long n, double inv_D) {
-    for (long long k = blockIdx.x * 256LL + threadIdx.x; k < n; k += (long long)gridDim.x * 256) {
-        const ff v = reinterpret_cast<const ff *>(a)[k];
-        a[k] = ((double)v.hi + (double)v.lo) * inv_D;
+// Packed interior -> caller grid.
+__global__ void __launch_bounds__(kBX) export_ff_kernel(const float *__restrict__ src, Grid g, double *u,
+                                                        long long ldu) {
+    const int i = blockIdx.x * kBX + threadIdx.x + 1;
+    if (i > g.Nx) return;
+    for (int j = blockIdx.y + 1; j <= g.Ny; j += gridDim.y) {
+        const long long k = ff_pos(g.idx(i, j));
+        u[(long long)(j - 1) * ldu + (i - 1)] = double_of(src[k]) + double_of(src[k + 2]);
     }
 }
 
-cudaError_t convert(double *a, long long n, bool to_ff, cudaStream_t s, double D = 1.0) {
-    const long long blocks = (n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096;
-    if (to_ff)
-        to_ff_kernel<<<(int)blocks, 256, 0, s>>>(a, n, D);
-    else
-        from_ff_kernel<<<(int)blocks, 256, 0, s>>>(a, n, 1.0 / D);
+// Zeroes the 16-byte pairs of both solution buffers that hold a ghost column: before the sweeps and
+// after them, as the pairs share their bytes differently in the two forms.  (The interior is
+// written before it is read, in either form, and so are the reflections of the 17-point stencil.)
+__global__ void __launch_bounds__(256) ghost_pairs_kernel(double *u0, double *u1, Grid g) {
+    const int j = (int)(blockIdx.x * 256 + threadIdx.x) - 1;
+    if (j > g.Ny + 2) return;
+    double *row[2] = {u0 + g.idx(1, j), u1 + g.idx(1, j)};
+    const int first = g.Nx & ~1;  // column offset of the first pair with a column past Nx
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        row[q][-2] = row[q][-1] = 0.0;
+        row[q][first] = row[q][first + 1] = 0.0;
+        if (first < g.Nx) row[q][first + 2] = row[q][first + 3] = 0.0;
+    }
+}
+
+cudaError_t ghost_pairs(const cj_plan *p, cudaStream_t s) {
+    ghost_pairs_kernel<<<(p->Ny + 4 + 255) / 256, 256, 0, s>>>(p->u0, p->u1, p->g64);
     return cudaGetLastError();
 }
 
@@ -267,42 +344,75 @@ cudaError_t convert(double *a, long long n, bool to_ff, cudaStream_t s, double D
 double ff_scale(int st) { return st == 9 ? 6.0 : 1.0; }
 double ff_centre(int st) { return st == 9 ? 20.0 : 4.0; }
 
+cudaError_t launch_sweep_ff(const cj_plan *p, FFArgs &a, cudaStream_t s) {
+    const Grid &g = p->g64;
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) sms = 152;
+    const long long np = (g.Nx + 1) / 2, threads = (long long)sms * kFFThreads;
+    // about 28 blocks an SM even out the sweep's end (at 10, a wave and a half, 9 points take 73.6 us on
+    // 4095 x 4001 against 67); on small grids a chunk's first rows should serve 4 rows (9-point
+    // 1024 x 1000: 5.85 us, at 2 rows 6.4) unless that leaves fewer than 7 blocks an SM
+    auto rows = [&](int per_sm) { return (np * g.Ny + threads * per_sm - 1) / (threads * per_sm); };
+    long long ty = rows(7) < 4 ? rows(7) : 4;
+    if (rows(28) > ty) ty = rows(28);
+    if (ty < 2) ty = 2;
+    if (ty > g.Ny) ty = g.Ny;
+    a.g = g;
+    a.ty = (int)ty;
+    a.chunks = (int)((g.Ny + ty - 1) / ty);
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)((np * a.chunks + kFFThreads - 1) / kFFThreads));
+    cfg.blockDim = dim3(kFFThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    void *args[] = {(void *)&a};
+    const void *fn = p->st == 5   ? (const void *)sweep_ff_kernel<5>
+                     : p->st == 9 ? (const void *)sweep_ff_kernel<9>
+                                  : (const void *)sweep_ff_kernel<17>;
+    return cudaLaunchKernelExC(&cfg, fn, args);
+}
+
 }  // namespace
 
 bool ff_sweeps_supported(const cj_plan *p) {
     return p && p->precision == CJ_FP64 && p->pattern == 0 && p->bc == CJ_BC_DIRICHLET0 && p->u1;
 }
 
-cudaError_t launch_sweeps_ff(const cj_plan *p, const double *const *bufs, long long first, long long count,
-                             int *cur_out, cudaStream_t s) {
-    *cur_out = 0;
-    if (count == 0) return cudaSuccess;  // no sweep: the iterate passes through unrounded
-    const long long n = p->g64.elems();
-    double *u[2] = {const_cast<double *>(bufs[0]), const_cast<double *>(bufs[1])};
-    double *b = const_cast<double *>(bufs[2]);
+cudaError_t launch_sweeps_ff(const cj_plan *p, const double *f, long long ldf, double *u, long long ldu,
+                             long long first, long long count, cudaStream_t s) {
+    float *buf[2] = {reinterpret_cast<float *>(p->u0), reinterpret_cast<float *>(p->u1)};
+    float *nb = reinterpret_cast<float *>(p->b);
     const double D = ff_scale(p->st);
-    cudaError_t e = convert(b, n, true, s, D);
-    if (e == cudaSuccess) e = convert(u[0], n, true, s);
-    if (e == cudaSuccess) e = convert(u[1], n, true, s);
-    int cur = 0, ty = 1;
-    const dim3 grid = ff_grid(p->g64, p->st, &ty);
+    const dim3 grid((p->Nx + kBX - 1) / kBX, p->Ny < 1024 ? p->Ny : 1024);
+    cudaError_t e = ghost_pairs(p, s);
+    if (e != cudaSuccess) return e;
+    if (p->st == 17)
+        import_ff_kernel<2><<<grid, kBX, 0, s>>>(f, ldf, u, ldu, nb, buf[0], p->g64, p->h2, D);
+    else
+        import_ff_kernel<1><<<grid, kBX, 0, s>>>(f, ldf, u, ldu, nb, buf[0], p->g64, p->h2, D);
+    e = cudaGetLastError();
+    int cur = 0;
     for (long long k = 0; k < count && e == cudaSuccess; ++k) {
         const double wk = p->w[(first + k) % p->M], wD = wk / D;
-        const FFWeights w{ff_of(wk), ff_of(wD), ff_of(1.0 - ff_centre(p->st) * wD)};
-        const ff *ui = reinterpret_cast<const ff *>(u[cur]);
-        ff *uo = reinterpret_cast<ff *>(u[cur ^ 1]);
-        const ff *bb = reinterpret_cast<const ff *>(b);
-        switch (p->st) {
-            case 5: sweep_ff_kernel<5><<<grid, kBX, 0, s>>>(ui, bb, uo, p->g64, ty, w); break;
-            case 9: sweep_ff_kernel<9><<<grid, kBX, 0, s>>>(ui, bb, uo, p->g64, ty, w); break;
-            default: sweep_ff_kernel<17><<<grid, kBX, 0, s>>>(ui, bb, uo, p->g64, ty, w); break;
-        }
-        e = cudaGetLastError();
+        FFArgs a{};
+        a.u = buf[cur];
+        a.nb = nb;
+        a.out = buf[cur ^ 1];
+        a.w = ff_of(wk);
+        a.wD = ff_of(wD);
+        a.c1 = ff_of(1.0 - ff_centre(p->st) * wD);
+        e = launch_sweep_ff(p, a, s);
         cur ^= 1;
     }
-    if (e == cudaSuccess) e = convert(u[0], n, false, s);
-    if (e == cudaSuccess) e = convert(u[1], n, false, s);
-    if (e == cudaSuccess) e = convert(b, n, false, s, D);
-    *cur_out = cur;
+    if (e == cudaSuccess) {
+        export_ff_kernel<<<grid, kBX, 0, s>>>(buf[cur], p->g64, u, ldu);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = ghost_pairs(p, s);
     return e;
 }
