@@ -116,6 +116,7 @@ class Engine {
         tile_cap_ = 0;
         d_.tiles = nullptr;
         d_.max_slots = max_slots;
+        d_.one = 1.0;
         ENG_TRY(cudaMallocHost(&h_status_, sizeof(SlotStatus) * max_slots), "engine status (host)");
         ENG_TRY(cudaMallocHost(&h_ntiles_, sizeof(int)), "engine tile count (host)");
         ENG_TRY(cudaMallocHost(&h_off_, sizeof(int) * (kEngLists + 1)), "engine item offsets (host)");

@@ -7,8 +7,11 @@
 // by the error-free TwoSum cascade (Sum2 of Ogita, Rump and Oishi); D L u_lo is added in
 // plain FP64.  This lifts the FP64 rounding floor of the relative residual (about
 // 2^-53 S ||u|| / ||b||, 5e-10 for the 9-point stencil on 4096^2), so the FP32 inner
-// cycles can drive the residual to 1e-10 and below.  Runs once per outer step, so it is a
-// plain one-thread-per-node kernel; the term order is fixed and equals the reference's.
+// cycles can drive the residual to 1e-10 and below.  Runs once per outer step, one thread per node;
+// the term order is fixed and equals the reference's.  Bound by the FP64 pipe: about 70 operations a
+// node for 9 points (FastTwoSums ordered on the integer pipe, the division by a constant in
+// three operations, the block sums two to an instruction; TwoSums, a division and separate
+// sums took 130): 9-point 1023^2 264 -> 148 us, the correction 31 -> 19 us (one GB300).
 // The inner cycle's type T is float (FP32 inner cycles) or double (FP64 inner cycles, whose
 // defect -R and correction e stay in FP64).
 #include "cj_internal.h"
@@ -22,15 +25,15 @@ __global__ void __launch_bounds__(kBX) defect_dd_kernel(const double *__restrict
                                                         const double *__restrict__ ul,
                                                         const double *__restrict__ b, Grid g,
                                                         T *rt, T *ez, Grid gt,
-                                                        double *partials) {
+                                                        double *partials, double one) {
     const int i = blockIdx.x * kBX + threadIdx.x + 1;
     double s2 = 0.0, mx = 0.0, u2 = 0.0;
     if (i <= g.Nx) {
         for (int j = blockIdx.y + 1; j <= g.Ny; j += gridDim.y) {
-            const double R = resid_dd<ST>(uh, ul, g, i, j, b[g.idx(i, j)]);
+            const double R = resid_dd<ST>(uh, ul, g, i, j, b[g.idx(i, j)], one);
             const double uc = uh[g.idx(i, j)];
             s2 = fma(R, R, s2);
-            mx = fmax(mx, fabs(R));
+            mx = max_abs(mx, R);
             u2 = fma(uc, uc, u2);
             rt[gt.idx(i, j)] = (T)(-R);
             store_node<(ST == 17 ? 2 : 1), T>(ez, gt, i, j, (T)0);
@@ -65,9 +68,9 @@ cudaError_t defect_dd_any(const cj_plan *p, const double *uh, const double *ul, 
                           const Grid &gt, cudaStream_t s) {
     const dim3 grid = node_grid(p->g64);
     switch (p->st) {
-        case 5: defect_dd_kernel<5, T><<<grid, kBX, 0, s>>>(uh, ul, p->b, p->g64, rt, e_zero, gt, p->partials); break;
-        case 9: defect_dd_kernel<9, T><<<grid, kBX, 0, s>>>(uh, ul, p->b, p->g64, rt, e_zero, gt, p->partials); break;
-        default: defect_dd_kernel<17, T><<<grid, kBX, 0, s>>>(uh, ul, p->b, p->g64, rt, e_zero, gt, p->partials); break;
+        case 5: defect_dd_kernel<5, T><<<grid, kBX, 0, s>>>(uh, ul, p->b, p->g64, rt, e_zero, gt, p->partials, 1.0); break;
+        case 9: defect_dd_kernel<9, T><<<grid, kBX, 0, s>>>(uh, ul, p->b, p->g64, rt, e_zero, gt, p->partials, 1.0); break;
+        default: defect_dd_kernel<17, T><<<grid, kBX, 0, s>>>(uh, ul, p->b, p->g64, rt, e_zero, gt, p->partials, 1.0); break;
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;

@@ -105,9 +105,9 @@ __global__ void __launch_bounds__(kEngThreads) eng_correct(EngineDev E) {
 }
 
 template <int ST>
-__device__ __forceinline__ double defect_value(const SlotDev &S, int i, int j) {
+__device__ __forceinline__ double defect_value(const SlotDev &S, int i, int j, double one) {
     const double bk = S.b[S.g64.idx(i, j)];
-    if (S.mode == CJ_FP32_INNER_DD) return resid_dd<ST>(S.u, S.ulo, S.g64, i, j, bk);
+    if (S.mode == CJ_FP32_INNER_DD) return resid_dd<ST>(S.u, S.ulo, S.g64, i, j, bk, one);
     auto U = [&](int di, int dj) { return S.u[S.g64.idx(i + di, j + dj)]; };
     return resid_direct<ST, double>(U, bk);
 }
@@ -123,12 +123,12 @@ __global__ void __launch_bounds__(kEngThreads) eng_defect(EngineDev E) {
         double s2 = 0.0, mx = 0.0, u2 = 0.0;
         if (i <= T.i1) {
             for (int j = T.j0; j <= T.j1; ++j) {
-                const double r = S.st == 5 ? defect_value<5>(S, i, j)
-                               : S.st == 9 ? defect_value<9>(S, i, j)
-                                           : defect_value<17>(S, i, j);
+                const double r = S.st == 5 ? defect_value<5>(S, i, j, E.one)
+                               : S.st == 9 ? defect_value<9>(S, i, j, E.one)
+                                           : defect_value<17>(S, i, j, E.one);
                 const double uc = S.u[S.g64.idx(i, j)];
                 s2 = fma(r, r, s2);
-                mx = fmax(mx, fabs(r));
+                mx = max_abs(mx, r);
                 u2 = fma(uc, uc, u2);
                 S.rt[S.g32.idx(i, j)] = (float)(-r);
                 if (S.st == 17)

@@ -60,6 +60,7 @@ struct EngineDev {
     int4 *items;           // register-tile items (slot, first column, first row, last row), by list
     int *item_off;         // kEngLists + 1 offsets of the lists in items
     SlotStatus *status;    // max_slots entries, refreshed by the advance kernel
+    double one;            // 1 (additions as fused multiply-adds)
 };
 
 // Streams and events of an engine's step: the lists' sweeps are branches of its graph, forked after

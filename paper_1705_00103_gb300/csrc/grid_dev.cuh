@@ -28,33 +28,39 @@ __device__ __forceinline__ void store_node(T *out, const Grid &g, int i, int j, 
 }
 
 
-// Block reduction of (sum, max, sum) into partials[3 * block].
-__device__ __forceinline__ void block_reduce3(double a, double m, double c, double *partials) {
-    __shared__ double sh[kBX / 32][3];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        a += __shfl_down_sync(0xffffffffu, a, o);
-        m = fmax(m, __shfl_down_sync(0xffffffffu, m, o));
-        c += __shfl_down_sync(0xffffffffu, c, o);
-    }
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0) {
-        sh[wid][0] = a;
-        sh[wid][1] = m;
-        sh[wid][2] = c;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double A = 0.0, Mx = 0.0, Cc = 0.0;
-        for (int k = 0; k < kBX / 32; ++k) {
-            A += sh[k][0];
-            Mx = fmax(Mx, sh[k][1]);
-            Cc += sh[k][2];
-        }
-        const long long blk = (long long)blockIdx.y * gridDim.x + blockIdx.x;
-        partials[3 * blk + 0] = A;
-        partials[3 * blk + 1] = Mx;
-        partials[3 * blk + 2] = Cc;
-    }
+// fmax(m, |r|) for m >= 0, a NaN r left out: on the bits, as the FP64 pipe's compare costs as much as
+// an addition.
+__device__ __forceinline__ double max_abs(double m, double r) {
+    const long long b = __double_as_longlong(r) & 0x7fffffffffffffffLL;
+    return b > __double_as_longlong(m) && b <= 0x7ff0000000000000LL ? __longlong_as_double(b) : m;
 }
 
+// Block reduction of (sum, max, sum) into partials[3 * block], m >= 0.  The two sums share each
+// step's addition: lanes 0..15 have the first and lanes 16..31 the second (a row of 128 nodes
+// would otherwise spend as many FP64 instructions here as on its residual).
+__device__ __forceinline__ void block_reduce3(double a, double m, double c, double *partials) {
+    __shared__ double sh[kBX / 32][3];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const double other = __shfl_xor_sync(0xffffffffu, lane < 16 ? c : a, 16);
+    double v = (lane < 16 ? a : c) + other;
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = max_abs(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (lane == 0) {
+        sh[wid][0] = v;
+        sh[wid][1] = m;
+    }
+    if (lane == 16) sh[wid][2] = v;
+    __syncthreads();
+    if (threadIdx.x < 3) {
+        const long long blk = (long long)blockIdx.y * gridDim.x + blockIdx.x;
+        double r = sh[0][lane];
+        if (threadIdx.x == 1) {
+            for (int k = 1; k < kBX / 32; ++k) r = max_abs(r, sh[k][1]);
+        } else {
+            for (int k = 1; k < kBX / 32; ++k) r += sh[k][lane];
+        }
+        partials[3 * blk + lane] = r;
+    }
+}

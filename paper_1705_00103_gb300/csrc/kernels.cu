@@ -35,7 +35,7 @@ struct ResidOp {
     int r2 = 0;
     __device__ __forceinline__ void operator()(int j, double r, double uc) {
         s2 = fma(r, r, s2);
-        mx = fmax(mx, fabs(r));
+        mx = max_abs(mx, r);
         u2 = fma(uc, uc, u2);
         if (rt) {
             rt[g32->idx(i, j)] = (float)(-r);
@@ -72,9 +72,10 @@ __global__ void __launch_bounds__(256) reduce_kernel(const double *__restrict__ 
                                                      int nparts, double *out) {
     __shared__ double sa[256], sm[256], sc[256];
     double a = 0.0, m = 0.0, c = 0.0;
-    for (int k = threadIdx.x; k < nparts; k += 256) {
+#pragma unroll 8
+    for (int k = threadIdx.x; k < nparts; k += 256) {  // (unrolled for its loads: the order of the sums stays)
         a += partials[3 * k + 0];
-        m = fmax(m, partials[3 * k + 1]);
+        m = max_abs(m, partials[3 * k + 1]);
         c += partials[3 * k + 2];
     }
     sa[threadIdx.x] = a;
@@ -84,7 +85,7 @@ __global__ void __launch_bounds__(256) reduce_kernel(const double *__restrict__ 
     for (int s = 128; s > 0; s >>= 1) {
         if (threadIdx.x < s) {
             sa[threadIdx.x] += sa[threadIdx.x + s];
-            sm[threadIdx.x] = fmax(sm[threadIdx.x], sm[threadIdx.x + s]);
+            sm[threadIdx.x] = max_abs(sm[threadIdx.x], sm[threadIdx.x + s]);
             sc[threadIdx.x] += sc[threadIdx.x + s];
         }
         __syncthreads();
@@ -111,7 +112,7 @@ __global__ void __launch_bounds__(kBX) import_kernel(const double *f, long long 
             double bk = h2 * fk;
             b[g.idx(i, j)] = bk;
             s = fma(bk, bk, s);
-            m = fmax(m, fabs(bk));
+            m = max_abs(m, bk);
             store_node<R, double>(u, g, i, j, uin[(long long)(j - 1) * ldu + (i - 1)]);
         }
     }

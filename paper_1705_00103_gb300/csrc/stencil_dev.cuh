@@ -197,86 +197,136 @@ __device__ __forceinline__ T resid_direct(F U, T bk) {
                                          Ar<T>::fm(Co<T>::d2(), Pm + Pp, Ar<T>::fm(Co<T>::cc17(), uC, -bk)))));
 }
 
+// s + e = a + b exactly: Knuth's TwoSum takes six FP64 operations; ordered by exponent on the integer
+// pipe, Dekker's FastTwoSum takes three and finds the same e.
 __device__ __forceinline__ void two_sum(double a, double b, double &s, double &e) {
-    double x = a + b;
-    double z = x - a;
-    e = (a - (x - z)) + (b - z);
+    const bool ordered =
+        ((unsigned)__double2hiint(a) & 0x7fffffffu) >= ((unsigned)__double2hiint(b) & 0x7fffffffu);
+    const double big = ordered ? a : b, small = ordered ? b : a;
+    const double x = a + b;
+    e = small - (x - big);
     s = x;
 }
 
+// The cascade S + E of TwoSums, adding c h for a power of two c = +-2^K.  Each TwoSum is ordered as
+// in two_sum above; c h is not formed: c goes into the fused multiply-adds, where its product is
+// exact.  (Terms below 2^-1018 may be ordered wrongly; what that can change is below 2^-1070.)
 struct Sum2 {
-    double S = 0.0, E = 0.0;
-    __device__ __forceinline__ void add(double t) {
-        double e;
-        two_sum(S, t, S, e);
-        E += e;
+    double S, E = 0.0;
+    double one;  // 1, as an argument: additions as fused multiply-adds
+    template <int K, bool NEG>
+    static __device__ __forceinline__ double c() {
+        return (NEG ? -1.0 : 1.0) * (double)(1 << K);
+    }
+    template <int K, bool NEG = false>
+    __device__ __forceinline__ void first(double h) {
+        S = fma(h, c<K, NEG>(), 0.0);
+    }
+    template <int K, bool NEG = false>
+    __device__ __forceinline__ void add(double h) {
+        const double cc = c<K, NEG>();
+        const double s = fma(h, cc, S);
+        const bool ordered = ((unsigned)__double2hiint(S) & 0x7fffffffu) >=
+                             ((unsigned)__double2hiint(h) & 0x7fffffffu) + ((unsigned)K << 20);
+        const double big = ordered ? S : h, small = ordered ? h : S;
+        const double cb = ordered ? 1.0 : cc, cs = ordered ? cc : 1.0;
+        const double z = fma(big, -cb, s);  // what of the smaller term s holds
+        E = fma(fma(small, cs, -z), one, E);
+        S = s;
     }
 };
 
-// Plain FP64 L u at node (i, j) in the evaluation order of the sweep kernels (b = 0).
-template <int ST>
-__device__ __forceinline__ double plain_L(const double *u, const Grid &g, int i, int j) {
-    auto U = [&](int di, int dj) { return u[g.idx(i + di, j + dj)]; };
-    return resid_direct<ST, double>(U, 0.0);
+// x / D, correctly rounded, for D = 6 or 72: x / D by the rounded reciprocal, corrected once by its
+// exact remainder (Markstein's theorem on division by fused multiply-adds); the division where the
+// remainder could underflow or nothing is finite.
+template <int D>
+__device__ __forceinline__ double div_const(double x) {
+    if (((unsigned)__double2hiint(x) >> 20 & 0x7ffu) - 128u > 1900u) return x / (double)D;
+    constexpr double y = 1.0 / D;
+    const double q = x * y;
+    return fma(fma(-(double)D, q, x), y, q);
 }
 
-// R = L (uh + ul) - bk at node (i, j), rounded to FP64 (term order as documented above).
+// FP64 L u at (i, j) of the padded grid u in resid_direct's order (b = 0), additions as fused
+// multiply-adds.
 template <int ST>
-__device__ __forceinline__ double resid_dd(const double *uh, const double *ul, const Grid &g,
-                                           int i, int j, double bk) {
-    auto H = [&](int di, int dj) { return uh[g.idx(i + di, j + dj)]; };
+__device__ __forceinline__ double plain_L(const double *u, const Grid &g, int i, int j, double one) {
+    using C = Co<double>;
+    const double *p = u + g.idx(i, j);
+    const long long P = g.pitch;
+    auto U = [&](int di, int dj) { return p[dj * P + di]; };
+    auto add = [&](double a, double b) { return fma(a, one, b); };
+    const double uC = U(0, 0);
+    const double s = add(add(U(-1, 0), U(1, 0)), add(U(0, -1), U(0, 1)));
+    if (ST == 5) return add(s, fma(C::c5(), uC, -0.0));
+    const double d = add(add(U(-1, -1), U(1, -1)), add(U(-1, 1), U(1, 1)));
+    if (ST == 9) return fma(C::ax9(), s, fma(C::dg9(), d, fma(C::cc9(), uC, -0.0)));
+    const double s2 = add(add(U(-2, 0), U(2, 0)), add(U(0, -2), U(0, 2)));
+    const double d2 = add(add(U(-2, -2), U(2, -2)), add(U(-2, 2), U(2, 2)));
+    return fma(C::a1(), s, fma(C::a2(), s2, fma(C::d1(), d, fma(C::d2(), d2, fma(C::cc17(), uC, -0.0)))));
+}
+
+// R = L (uh + ul) - bk at node (i, j), rounded to FP64 (term order as documented above).  one: 1.
+template <int ST>
+__device__ __forceinline__ double resid_dd(const double *uh, const double *ul, const Grid &g, int i, int j, double bk,
+                                           double one) {
+    const double *p = uh + g.idx(i, j);
+    const long long P = g.pitch;
+    auto H = [&](int di, int dj) { return p[dj * P + di]; };
     const double uC = H(0, 0);
     Sum2 s;
-    double D;
+    s.one = one;
+    constexpr int D = ST == 5 ? 1 : ST == 9 ? 6 : 72;
     if (ST == 5) {
-        D = 1.0;
-        s.add(H(-1, 0));
-        s.add(H(1, 0));
-        s.add(H(0, -1));
-        s.add(H(0, 1));
-        s.add(-4.0 * uC);
-        s.add(-bk);
+        s.first<0>(H(-1, 0));
+        s.add<0>(H(1, 0));
+        s.add<0>(H(0, -1));
+        s.add<0>(H(0, 1));
+        s.add<2, true>(uC);
+        s.add<0, true>(bk);
     } else if (ST == 9) {
-        D = 6.0;
-        s.add(4.0 * H(-1, 0));
-        s.add(4.0 * H(1, 0));
-        s.add(4.0 * H(0, -1));
-        s.add(4.0 * H(0, 1));
-        s.add(H(-1, -1));
-        s.add(H(1, -1));
-        s.add(H(-1, 1));
-        s.add(H(1, 1));
-        s.add(-16.0 * uC);
-        s.add(-4.0 * uC);
-        s.add(-4.0 * bk);
-        s.add(-2.0 * bk);
+        s.first<2>(H(-1, 0));
+        s.add<2>(H(1, 0));
+        s.add<2>(H(0, -1));
+        s.add<2>(H(0, 1));
+        s.add<0>(H(-1, -1));
+        s.add<0>(H(1, -1));
+        s.add<0>(H(-1, 1));
+        s.add<0>(H(1, 1));
+        s.add<4, true>(uC);
+        s.add<2, true>(uC);
+        s.add<2, true>(bk);
+        s.add<1, true>(bk);
     } else {
-        D = 72.0;
-        s.add(64.0 * H(-1, 0));
-        s.add(64.0 * H(1, 0));
-        s.add(64.0 * H(0, -1));
-        s.add(64.0 * H(0, 1));
-        s.add(-4.0 * H(-2, 0));
-        s.add(-4.0 * H(2, 0));
-        s.add(-4.0 * H(0, -2));
-        s.add(-4.0 * H(0, 2));
-        s.add(16.0 * H(-1, -1));
-        s.add(16.0 * H(1, -1));
-        s.add(16.0 * H(-1, 1));
-        s.add(16.0 * H(1, 1));
-        s.add(-H(-2, -2));
-        s.add(-H(2, -2));
-        s.add(-H(-2, 2));
-        s.add(-H(2, 2));
-        s.add(-256.0 * uC);
-        s.add(-32.0 * uC);
-        s.add(-8.0 * uC);
-        s.add(-4.0 * uC);
-        s.add(-64.0 * bk);
-        s.add(-8.0 * bk);
+        s.first<6>(H(-1, 0));
+        s.add<6>(H(1, 0));
+        s.add<6>(H(0, -1));
+        s.add<6>(H(0, 1));
+        s.add<2, true>(H(-2, 0));
+        s.add<2, true>(H(2, 0));
+        s.add<2, true>(H(0, -2));
+        s.add<2, true>(H(0, 2));
+        s.add<4>(H(-1, -1));
+        s.add<4>(H(1, -1));
+        s.add<4>(H(-1, 1));
+        s.add<4>(H(1, 1));
+        s.add<0, true>(H(-2, -2));
+        s.add<0, true>(H(2, -2));
+        s.add<0, true>(H(-2, 2));
+        s.add<0, true>(H(2, 2));
+        s.add<8, true>(uC);
+        s.add<5, true>(uC);
+        s.add<3, true>(uC);
+        s.add<2, true>(uC);
+        s.add<6, true>(bk);
+        s.add<3, true>(bk);
     }
-    const double Llo = plain_L<ST>(ul, g, i, j);
-    return (s.S + (s.E + D * Llo)) / D;
+    const double Llo = plain_L<ST>(ul, g, i, j, one);
+    const double t = fma(s.S, one, fma(s.E, one, (double)D * Llo));
+    if constexpr (D == 1)
+        return t;
+    else
+        return div_const<D>(t);
 }
 
 }  // namespace
