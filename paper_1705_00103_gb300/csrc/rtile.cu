@@ -89,15 +89,20 @@ RtTiles rt_tiles(const RtKernel &K, int R, int Nx, int Ny, int k) {
 
 // The shape with the shortest modelled launch of k sweeps, and that time in us: a fixed part (launch,
 // first load, last store), and for the SM with the most tiles the sweeps of its staged rows (row_us
-// each) and their loads and stores at its share of the HBM rate (0.032 us a row; 0.012 from the L2),
-// which overlap in part, as the blocks of an SM drift apart: the root of the sum of squares.
+// each) and their loads and stores at its share of the HBM rate (0.032 us a row; 0.012 from the L2, and
+// in between where e, r and the output take 20 to 60 MB of its 129), which overlap in part, as the blocks
+// of an SM drift apart: the root of the sum of squares.  Over 34 sizes from 150 to 8192 a side the depth
+// and shape chosen are within 1.2 / 0.4 / 0.6 % of the fastest on average (5 / 9 / 17 points) and
+// within 13 / 6 / 8 % at worst; with one step from L2 to HBM at 100 MB the worst was 38 % (17-point 3000
+// x 2700: 14.4 us a sweep, now 10.4; 9-point 2048^2: 3.23, now 2.84).
 // Modelled / measured us (9-point unless said): 400^2, 8 x 4 rows, k = 8: 4.1 / 4.3; 640^2, 8 x 8,
 // k = 16: 9.3 / 9.6; 1500^2, 12 x 8, k = 8: 12.8 / 13.5; 4096^2, 14 x 8, k = 4: 46.5 / 47.5, k = 8:
 // 78 / 73; 8192^2, 16 x 8, k = 8: 294 / 262; 17-point 8192^2, 14 x 8, k = 2: 174 / 169, k = 4: 315 / 275.
 int rt_choose(int st, int Nx, int Ny, int k, double *us) {
     const RtKernels &S = rt_kernels(st);
     const int R = st == 17 ? 2 : 1, sms = rt_sms();
-    const double mem_us = 12.0 * Nx * Ny > 100e6 ? 0.032 : 0.012;  // e, r and the output against the L2
+    const double hbm = std::fmin(std::fmax((12e-6 * Nx * Ny - 20.0) / 40.0, 0.0), 1.0);
+    const double mem_us = 0.012 + 0.020 * hbm;
     int best = 0;
     *us = 1e300;
     for (int i = 0; i < S.n; ++i) {
