@@ -18,9 +18,13 @@
 
 namespace {
 
-// Sweep launches per engine step, and steps per captured graph: a replay advances a slot by up to
-// 256 sweeps (8 per launch; 17 points: 128).
-constexpr int kSweepsPerStep = 8;
+// Sweep launches per captured graph: a replay advances a slot by up to 256 sweeps (8 per launch; 17
+// points: 128).  They are one engine step, or kShortSteps where every inner cycle at hand ends
+// within fewer launches than that: a step's five other kernels cost about 20 us, against 10 us a
+// launch (measured, steps of 8 launches -> 32: 32 problems of 64 .. 1024 a side 17.3 -> 16.4 ms, 8 served
+// requests of 32 .. 300 4.7 -> 4.2 ms), but a slot waits for its step's end once its cycle has ended
+// (16 problems of 8 .. 24 a side, cycles of 4 to 8 launches: 1.84 ms with 8, 2.03 with 32).
+constexpr int kSweepsPerGraph = 32, kShortSteps = 4;
 // Shorter side from which the autotuner times depth 4 of 5 and 9 points.
 constexpr int kEngDeepMinSide = 512;
 
@@ -307,7 +311,7 @@ class Engine {
         for (int k = 0; k < replays; ++k) ENG_TRY(cudaGraphLaunch(gexec_, s_), "graph launch");
         int nlists = 0;
         for (int l = 0; l < kEngBranches; ++l) nlists += (int)(lists_ >> l & 1u);
-        launches_ += (long long)replays * steps_per_graph_ * (5 + nlists * kSweepsPerStep);
+        launches_ += (long long)replays * (steps_per_graph_ * 5 + nlists * kSweepsPerGraph);
         ENG_TRY(cudaMemcpyAsync(h_status_, d_.status, sizeof(SlotStatus) * max_slots_,
                                 cudaMemcpyDeviceToHost, s_), "status readback");
         ENG_TRY(cudaStreamSynchronize(s_), "step sync");
@@ -388,11 +392,16 @@ class Engine {
     }
 
     cj_status capture() {
+        long long cycle = 0;  // launches of the longest inner cycle
+        for (int q = 0; q < max_slots_; ++q)
+            if (used_[q]) cycle = std::max(cycle, host_[q].M_in / host_[q].depth);
+        steps_per_graph_ = cycle >= kSweepsPerGraph ? 1 : kShortSteps;
         cudaGraph_t g = nullptr;
         ENG_TRY(cudaStreamBeginCapture(s_, cudaStreamCaptureModeThreadLocal), "begin capture");
         cudaError_t err = cudaSuccess;
         for (int k = 0; k < steps_per_graph_ && err == cudaSuccess; ++k)
-            err = eng_launch_step(d_, grid_tiles_, grid_slots_, lists_, rt_blocks_, br_, kSweepsPerStep, s_);
+            err = eng_launch_step(d_, grid_tiles_, grid_slots_, lists_, rt_blocks_, br_, kSweepsPerGraph / steps_per_graph_,
+                                  s_);
         cudaError_t e2 = cudaStreamEndCapture(s_, &g);
         if (err == cudaSuccess) err = e2;
         if (err == cudaSuccess) err = cudaGraphInstantiate(&gexec_, g, 0);
@@ -448,7 +457,7 @@ class Engine {
 
     int dev_ = 0, max_slots_ = 0, grid_tiles_ = 0, grid_slots_ = 0, rt_blocks_ = 0;
     unsigned lists_ = 0;
-    int steps_per_graph_ = 4;
+    int steps_per_graph_ = 1;
     EngineBranches br_;
     cudaStream_t s_ = nullptr;
     EngineDev d_{};
@@ -889,7 +898,7 @@ cj_status cj_autotune_engine(int Nx, int Ny, cj_stencil st, int *tile_rows, int 
     // candidates, the default (32 rows, depth 1) first so that it wins ties
     const int tys[9] = {32, 16, 64, 32, 16, 64, 32, 16, 64};
     const int dps[9] = {1, 1, 1, 2, 2, 2, 4, 4, 4};
-    const int kReplays = 8;  // 8 replays x 8 steps x 4 sweep launches
+    const int kReplays = 8;  // of 32 sweep launches each
     double rate[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
     // a synthetic problem of this class: f constant (every byte 0x3F, about 4.8e-4), u0 = 0,
     // a tolerance no slot reaches within the timed replays
