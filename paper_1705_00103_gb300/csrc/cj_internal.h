@@ -134,6 +134,8 @@ cudaError_t launch_sweeps_ff(const cj_plan *p, const double *f, long long ldf, d
 // CTAs of the cluster the plan's solve fits in (0: not eligible: not plain FP64 on the paper's
 // stencils, more than 2^14 nodes, or no cluster launch on this device)
 int cluster_solve_size(const cj_plan *p);
+// false where the captured sweeps of the plan are faster (p->cluster_C > 0)
+bool cluster_solve_pays(const cj_plan *p);
 // the solve of p->u0 against p->b (imported, red[3..4] set) with the plan's weights table w_dev;
 // res_dev[0..5] = status, sweeps, cycles, rho, rinf, fl
 cudaError_t launch_cluster_solve(const cj_plan *p, double *res_dev, cudaStream_t s);

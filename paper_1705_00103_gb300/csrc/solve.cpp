@@ -726,6 +726,7 @@ cj_status cj_plan_create(int Nx, int Ny, cj_stencil st, cj_bc bc, double tol,
     if (e == cudaSuccess && graph) e = make_sweep_graph(p);
     if (e == cudaSuccess && (o.launch == 0 || o.launch == 3)) {
         p->cluster_C = cluster_solve_size(p);
+        if (o.launch == 0 && p->cluster_C > 0 && p->graph && !cluster_solve_pays(p)) p->cluster_C = 0;
         if (p->cluster_C > 0 && !p->w_dev) {
             e = cudaMalloc((void **)&p->w_dev, sizeof(double) * (size_t)p->M);
             if (e == cudaSuccess)
