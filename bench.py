@@ -52,9 +52,9 @@ STENCIL = 9
 TOL = 1e-10
 METRIC = "CJM time-to-1e-10 residual & Gupdates/s vs plain FP64; HBM GB/s; p50/p99 latency"
 UNIT = "Gupdates/s"
-# FP64 instructions per grid-point update of the sweep (9-point tree: 4 pair/group sums,
-# 3 coefficient fmas, 1 update fma) and algorithmic bytes (read u and b, write u')
-FP64_OPS_PER_UPDATE = {5: 6, 9: 8, 17: 14}
+# FP64-pipe instructions per grid-point update of the sweep (9 points: 3 coefficient fmas and 1
+# update fma; its 4 pair and group sums run on the integer pipe) and algorithmic bytes (read u and b, write u')
+FP64_OPS_PER_UPDATE = {5: 3, 9: 4, 17: 6}
 BYTES_PER_UPDATE_FP64 = 24
 # FP64 issue peak: 1.25 TFLOP/s nominal = 2 FP64 FMA per SM per clock x 152 SMs x 2.07 GHz
 FP64_PEAK_TOPS = 2 * 152 * 2.07e9 / 1e12
@@ -183,7 +183,7 @@ class ClockSampler:
 
 # ----------------------------------------------------------------- traffic record
 
-KERNEL_SOURCES = ("kernels.cu", "stencil_dev.cuh", "grid_dev.cuh")
+KERNEL_SOURCES = ("sweep64.cu", "stencil_dev.cuh", "grid_dev.cuh")
 # sources of the FP32 register-tile kernel (temporal blocking)
 RTILE_SOURCES = ("rtile.cu", "rtile_dev.cuh", "fold_dev.cuh", "grid_dev.cuh", "stencil_dev.cuh", "cj_internal.h")
 # FP32 operations per 9-point update of the register-tile kernel (second-difference form):
@@ -197,12 +197,12 @@ FP32_ISSUE_PEAK_TOPS = 4 * 32 * 152 * 2.07e9 / 1e12
 
 
 # sources of the float-float sweep kernel
-FF_SOURCES = ("ff.cu", "grid_dev.cuh", "stencil_dev.cuh", "cj_internal.h")
+FF_SOURCES = ("ff.cu", "cj_internal.h")
 # FP32 instructions per 9-point update of the float-float sweep in its scaled form
 # u' = c1 u + (w/6) (4 a + d - 6 b): 7 float-float adds (11 each: TwoSum 6, low parts 2,
-# FastTwoSum 3; the row pair, the vertical pair, a, d, 4 a + d, - 6 b and the final sum), the
-# exact scaling by 4 (2) and 2 TwoProduct multiplies (7 each)
-FF_OPS_PER_UPDATE_9 = 7 * 11 + 2 + 2 * 7
+# FastTwoSum 3; the row pair, the vertical pair, a, d, 4 a + d with the scaling inside its
+# multiply-adds, - 6 b and the final sum) and 2 TwoProduct multiplies (7 each)
+FF_OPS_PER_UPDATE_9 = 7 * 11 + 2 * 7
 
 
 def kernel_digest(sources=KERNEL_SOURCES) -> str:
@@ -334,13 +334,14 @@ def run_cj(args):
     avg_sweep_s = sweep_s / sweeps
     ops = FP64_OPS_PER_UPDATE[STENCIL] * N_GRID * N_GRID
     achieved = ops / avg_sweep_s / 1e12
-    traffic = traffic_per_launch("sweep_kernel_9_f64_4096")
+    traffic = traffic_per_launch("sweep64_9_4096")
     hbm_gbs = BYTES_PER_UPDATE_FP64 * N_GRID * N_GRID / avg_sweep_s / 1e9
     roofline = {"bound": "alu", "achieved": achieved, "peak": peaks["fp64_tfma_s"], "unit": "TFP64op/s",
                 "frac": achieved / peaks["fp64_tfma_s"], "traffic": traffic,
-                "kernel": "sweep_kernel<9,double>", "avg_launch_us": avg_sweep_s * 1e6,
-                "peak_note": "FP64 FMA issue rate measured on this GPU by cj_issue_peaks (the sweep issues "
-                             "every FP64 operation as an FMA: 8 per 9-point update); of measured",
+                "kernel": "sweep64_kernel<9>", "avg_launch_us": avg_sweep_s * 1e6,
+                "peak_note": "FP64 FMA issue rate measured on this GPU by cj_issue_peaks (4 operations of a "
+                             "9-point update are left on the FP64 pipe, its other 4 additions run on the "
+                             "integer pipe where every lane of a warp can); of measured",
                 "peak_nominal": FP64_PEAK_TOPS, "frac_of_nominal": achieved / FP64_PEAK_TOPS,
                 "hbm": {"achieved_gbs": hbm_gbs, "peak_gbs": hbm_peak, "frac": hbm_gbs / hbm_peak,
                         "bytes_per_update": BYTES_PER_UPDATE_FP64, "peak_note": hbm_note},
@@ -515,8 +516,8 @@ def fp32_sweep_roofline(cj, stream, peaks, launches: int = 64) -> dict:
 def ff_sweep_roofline(cj, f, stream, peaks, sweeps: int = 64) -> dict:
     """The float-float sweep (cj_sweeps_ff: the FP64 sweep's expression in pairs of floats on the
     FP32 pipe) beside the bit-exact FP64 sweep, on the 4096^2 9-point grid: `sweeps` sweeps of
-    the plan's cycle in one call each (the float-float call includes its 6 in-place conversions
-    of the three FP64 grids), timed with CUDA events on the launching stream; and its largest
+    the plan's cycle in one call each (with its import, which converts to float-float, and its
+    export), timed with CUDA events on the launching stream; and its largest
     deviation from the FP64 kernel over the first sweep from a random iterate, relative to the
     per-sweep scale max|u| + |w| (9 max|u| + max|b|)."""
     import torch
@@ -566,7 +567,7 @@ def ff_sweep_roofline(cj, f, stream, peaks, sweeps: int = 64) -> dict:
             "dev_weight_index": k,
             "note": "FP64-accuracy (48-bit float-float) sweep, not bit-equal to the FP64 sweep; per-sweep "
                     "deviation held to 1e-12 of the sweep scale by the parity tests; timings include the "
-                    "in-place conversions of the three grids, amortised over the call's sweeps"}
+                    "converting import and export, amortised over the call's sweeps"}
 
 
 def highorder_key(cj, stream, steps: int = 1) -> dict:

@@ -6,7 +6,8 @@
     python -m paper_1705_00103_gb300.profile_sweeps --stencil 9 --n 4096 --precision ff --count 16
     python -m paper_1705_00103_gb300.profile_sweeps --stencil 9 --n 1024 --batch 24 --depth 4
 
-Inputs are zero grids of the given size (the sweep's cost does not depend on the values);
+Inputs are zero grids of the given size (FP64 sweeps of them take every row's additions on the FP64
+pipe: twice the time of a smooth iterate; the others' cost does not depend on the values);
 three FP64 grids of 4096^2 (400 MB) exceed the 129 MB L2.
 """
 from __future__ import annotations
@@ -69,12 +70,12 @@ def main(argv=None):
             e0 = torch.cuda.Event(enable_timing=True)
             e1 = torch.cuda.Event(enable_timing=True)
             e0.record()
-            fn(a.time)
+            fn(a.time + 1)
             e1.record()
             torch.cuda.synchronize()
             ms = e0.elapsed_time(e1)
             e0.record()
-            fn(0)
+            fn(1)
             e1.record()
             torch.cuda.synchronize()
             per = (ms - e0.elapsed_time(e1)) / a.time

@@ -43,3 +43,33 @@ def test_isolated_nodes(st, Nx, Ny):
             ref = orc.sweep(st, u, f, w[k])
             rel = np.where(scale < 2.0 ** -70, 2.0 ** -21, 2.0 ** -42)
             assert np.all(np.abs(ud.cpu().numpy() - ref) <= rel * scale * (1.0 + abs(w[k]) * c))
+
+
+@pytest.mark.parametrize("st", [5, 9, 17])
+@pytest.mark.parametrize("Nx,Ny", [(60, 41), (61, 40), (1, 1), (2, 3), (127, 130)])
+def test_plan_after_float_float_sweeps(st, Nx, Ny):
+    """FP64 calls of a plan give the oracle's bits after float-float sweeps have used its buffers in
+    their own form (an odd number of sweeps and an even one)."""
+    import torch
+
+    import paper_1705_00103_gb300 as cj
+    rng = np.random.default_rng(Nx + 10 * st)
+    f, u = rng.standard_normal((Ny, Nx)), rng.standard_normal((Ny, Nx))
+    b = orc.scale_rhs(f)
+    fd = torch.from_numpy(f).cuda()
+    with cj.Plan(Nx, Ny, st, 1e-6) as p:
+        w = p.info()["w"]
+        ref = u
+        for k in range(3):
+            ref = orc.sweep(st, ref, b, w[k % len(w)])
+        for count in (1, 2):
+            cj.cj_sweeps_ff(p.handle, fd, torch.from_numpy(u.copy()).cuda(), 0, count)
+            ud = torch.from_numpy(u.copy()).cuda()
+            cj.cj_sweeps(p.handle, fd, ud, 0, 3)
+            np.testing.assert_array_equal(ud.cpu().numpy(), ref)
+            cj.cj_sweeps_ff(p.handle, fd, torch.from_numpy(u.copy()).cuda(), 0, count)
+            ud = torch.zeros((Ny, Nx), dtype=torch.float64, device="cuda")
+            res = cj.cj_solve(p.handle, fd, ud)
+            want = orc.solve(st, f, 1e-6)
+            assert res["sweeps"] == want["sweeps"]
+            np.testing.assert_array_equal(ud.cpu().numpy(), want["u"])
