@@ -188,6 +188,7 @@ class Engine {
         long long M_in;
         cj_status st = plan(sp, &kmin, &kmax, &M_in);
         if (st != CJ_OK) return st;
+        if (!(lists_ >> list_of(sp) & 1u)) return CJ_ERR_INVALID_ARG;
         const size_t bytes = slot_bytes(sp, M_in);
         char *base = nullptr;
         ENG_TRY(cudaMallocAsync((void **)&base, bytes, s_), "slot memory");
@@ -197,7 +198,6 @@ class Engine {
         S.Ny = sp.Ny;
         S.st = sp.st;
         S.mode = sp.mode;
-        if (!(lists_ >> list_of(sp) & 1u)) return CJ_ERR_INVALID_ARG;
         S.depth = (int)std::min<long long>(sp.depth, M_in);
         S.plain = list_of(sp) == kEngPlain;
         S.ty = sp.ty;
@@ -829,10 +829,12 @@ extern "C" {
 cj_status cj_solve_batch(const cj_problem *problems, int n, void *stream, cj_result *results) {
     if (!problems || n < 1 || !results) return CJ_ERR_INVALID_ARG;
     unsigned lists = 0;
+    std::vector<Spec> specs;  // read from the tuning table once: another thread may be tuning
     for (int k = 0; k < n; ++k) {
         cj_status st = check_problem(problems[k]);
         if (st != CJ_OK) return st;
-        lists |= 1u << Engine::list_of(spec_of(problems[k]));
+        specs.push_back(spec_of(problems[k]));
+        lists |= 1u << Engine::list_of(specs[k]);
     }
     auto t0 = Clock::now();
     Engine eng;
@@ -846,7 +848,7 @@ cj_status cj_solve_batch(const cj_problem *problems, int n, void *stream, cj_res
     long long max_steps = 0;
     for (int k = 0; k < n; ++k) {
         const cj_problem &pr = problems[k];
-        const Spec sp = spec_of(pr);
+        const Spec &sp = specs[k];
         st = eng.admit(sp, pr.f, pr.ld_f, pr.u, pr.ld_u, pr.u, pr.ld_u, &slot[k]);
         if (st != CJ_OK) {
             cudaEventDestroy(ev);
