@@ -363,10 +363,10 @@ typedef struct {
                                FP64 floor (about 2^-53 S / (c kmin)) is within 4x of tol */
     double tol;
     int inner_cycle;        /* 0 = the planner's choice */
-    int temporal_depth;     /* FP32 sweeps per sweep launch (temporal blocking), 1..8; 0 = 8 (17
-                               points: 4), or 1 where cj_autotune_engine measured one sweep per
-                               launch as the fastest for the size class.  Depths of 2 and more run
-                               the register tiles of cj_sweeps_f32 over the problem's tiles */
+    int temporal_depth;     /* FP32 sweeps per sweep launch (temporal blocking), 1..8; 0 = the
+                               depth cj_autotune_engine recorded for the size class, else 8 (17
+                               points: 4).  Depths of 2 and more run the register tiles of
+                               cj_sweeps_f32 over the problem's tiles */
     long long max_sweeps;   /* 0 = 64 inner cycles */
     const double *f;        /* device, Ny x ld_f, unscaled right-hand side */
     long long ld_f;
@@ -384,7 +384,7 @@ typedef struct {
  * and replayed until every slot has finished; finished problems leave the tile list; tile
  * rows (16/32/64; of the outer steps' kernels) come from cj_autotune_engine's table for the size
  * class when it has an entry.  The sweeps run on register tiles, eight per launch (17 points:
- * four), the problems of one stencil and tile shape in one branch of the step's graph.  A problem's arithmetic does not depend on its batch-mates.  results[k] receives problem k's outcome (status per
+ * four) unless the table or the problem names another depth, the problems of one stencil and tile shape in one branch of the step's graph.  A problem's arithmetic does not depend on its batch-mates.  results[k] receives problem k's outcome (status per
  * problem; seconds and launches are those of the whole batch).  Orders itself after the
  * work already on `stream` and makes `stream` wait for it; blocks until done.  Returns
  * CJ_OK, or CJ_ERR_TIMEOUT if a problem did not finish within its sweep budget's steps.
@@ -401,17 +401,18 @@ typedef struct {
 } cj_server_stats_t;
 
 /*
- * cj_autotune_engine -- tile rows (16, 32 or 64; 128 columns) and FP32 temporal depth (1, 2 or 4)
- * of the batched / served engine for a stencil and size class (grids within a factor 2 per side),
- * picked by timing the engine loaded with copies of a synthetic problem of Nx x Ny nodes (as
- * many as give the device ~8 tiles per SM, up to 256 and 2^24 nodes) at every combination, and
- * recorded in a per-process table that cj_solve_batch and the server use for problems of that
- * class (the server takes the tile rows only; a depth of 2 or 4 means fused sweeps, which the batch
- * runs at the register tiles' own depth; an explicit temporal_depth overrides it).  Depth 4 of 5 and
- * 9 points is a candidate only when both sides are at least 512 (its rate is reported as 0 below).
+ * cj_autotune_engine -- tile rows (16, 32 or 64; 128 columns) and FP32 temporal depth of the batched
+ * / served engine for a stencil and size class (grids within a factor 2 per side), picked by timing
+ * the engine loaded with copies of a synthetic problem of Nx x Ny nodes (as many as give the device
+ * ~8 tiles per SM, up to 256 and 2^24 nodes) at every combination of rows and depths 1, 2 and 4, and
+ * at the default depth (cj_problem's 0).  The fastest is recorded, as it was timed, in a per-process
+ * table that cj_solve_batch and the server use for problems of that class (the server takes the tile
+ * rows only; an explicit temporal_depth overrides the depth).  Depth 4 of 5 and 9 points is a
+ * candidate only when both sides are at least 512 (its rate is reported as 0 below).
  * Not a method of the paper: a runtime choice of this library.  Synchronous; allocates an Nx x Ny
  * FP64 grid and the engine's slots while it runs.
- *   tile_rows, depth: the choice (may be NULL);
+ *   tile_rows, depth: the fastest of the nine combinations (may be NULL), which is the recorded choice
+ *     unless the default depth was faster still;
  *   gupd: host array of 9 (may be NULL): measured Gupdates/s, tile rows 16/32/64 (major) x
  *     depth 1/2/4.
  * Returns CJ_ERR_INVALID_ARG for a bad size or stencil.

@@ -562,8 +562,9 @@ class Plan:
 
 
 def cj_autotune_engine(Nx: int, Ny: int, st: int) -> dict:
-    """Times the batched engine at tile rows 16/32/64 x depth 1/2/4 for this stencil and size
-    class and records the fastest for cj_solve_batch and the server (see cj.h)."""
+    """Times the batched engine at tile rows 16/32/64 x depth 1/2/4 and at its default depth for this
+    stencil and size class and records the fastest for cj_solve_batch and the server; returns the
+    fastest of the nine (see cj.h)."""
     ty, d = ctypes.c_int(), ctypes.c_int()
     g = (ctypes.c_double * 9)()
     rc = _lib().cj_autotune_engine(Nx, Ny, st, ctypes.byref(ty), ctypes.byref(d), g)

@@ -25,7 +25,8 @@ namespace {
 // requests of 32 .. 300 4.7 -> 4.2 ms), but a slot waits for its step's end once its cycle has ended
 // (16 problems of 8 .. 24 a side, cycles of 4 to 8 launches: 1.84 ms with 8, 2.03 with 32).
 constexpr int kSweepsPerGraph = 32, kShortSteps = 4;
-// Shorter side from which the autotuner times depth 4 of 5 and 9 points.
+// Shorter side from which the autotuner times and reports depth 4 of 5 and 9 points (the default depth
+// is timed at every size).
 constexpr int kEngDeepMinSide = 512;
 
 using Clock = std::chrono::steady_clock;
@@ -294,18 +295,19 @@ class Engine {
         return CJ_OK;
     }
 
+    // Brings the device's tile and item tables in line with the slots.
+    cj_status upload() { return tiles_dirty_ ? upload_tiles() : CJ_OK; }
+
     // Runs `replays` graph replays of the engine steps, then refreshes the host status.
     cj_status run(int replays) {
-        if (tiles_dirty_) {
-            cj_status st = upload_tiles();
-            if (st != CJ_OK) return st;
-        }
+        cj_status st = upload();
+        if (st != CJ_OK) return st;
         if (!gexec_) {
-            cj_status st = capture();
+            st = capture();
             if (st != CJ_OK) return st;
         }
         if (tile_grid_ && grids_dirty_) {
-            cj_status st = set_tile_grid();
+            st = set_tile_grid();
             if (st != CJ_OK) return st;
         }
         for (int k = 0; k < replays; ++k) ENG_TRY(cudaGraphLaunch(gexec_, s_), "graph launch");
@@ -491,7 +493,7 @@ int auto_mode(int st, int Nx, int Ny, double tol) {
 }
 
 // Engine tile rows and temporal depth per (stencil, size class) recorded by
-// cj_autotune_engine; 0 = not tuned (tile rows 32, depth 1).
+// cj_autotune_engine, as it timed them; 0 = not tuned (kEngTYDefault rows, eng_default_depth).
 struct EngineTune {
     int ty, depth;
 };
@@ -524,8 +526,7 @@ Spec spec_of(const cj_problem &pr) {
     sp.mode = pr.precision ? pr.precision : auto_mode(pr.st, pr.Nx, pr.Ny, pr.tol);
     sp.inner_cycle = pr.inner_cycle;
     EngineTune t = engine_tuned(pr.st, pr.Nx, pr.Ny);
-    // a measured preference for one sweep per launch stands; fused sweeps run at the tiles' own depth
-    sp.depth = pr.temporal_depth ? pr.temporal_depth : (t.depth == 1 ? 1 : eng_default_depth(pr.st));
+    sp.depth = pr.temporal_depth ? pr.temporal_depth : (t.depth ? t.depth : eng_default_depth(pr.st));
     sp.ty = t.ty ? t.ty : kEngTYDefault;
     sp.max_sweeps = pr.max_sweeps;
     return sp;
@@ -897,13 +898,14 @@ cj_status cj_solve_batch(const cj_problem *problems, int n, void *stream, cj_res
 cj_status cj_autotune_engine(int Nx, int Ny, cj_stencil st, int *tile_rows, int *depth, double *gupd) {
     if (Nx < 1 || Ny < 1 || Nx > (1 << 20) || Ny > (1 << 20)) return CJ_ERR_INVALID_ARG;
     if (st != CJ_ST5 && st != CJ_ST9 && st != CJ_ST17) return CJ_ERR_INVALID_ARG;
-    // candidates, the default (32 rows, depth 1) first so that it wins ties
+    // the reported candidates, and after them the default depth at 32 rows, which an untuned problem
+    // runs, and at the rows the nine favour
     const int tys[9] = {32, 16, 64, 32, 16, 64, 32, 16, 64};
     const int dps[9] = {1, 1, 1, 2, 2, 2, 4, 4, 4};
-    const int kReplays = 8;  // of 32 sweep launches each
+    const int kReplays = 8;  // of 32 sweep launches each, or until every copy has ended
     double rate[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
     // a synthetic problem of this class: f constant (every byte 0x3F, about 4.8e-4), u0 = 0,
-    // a tolerance no slot reaches within the timed replays
+    // a tolerance few slots reach within the timed replays
     const size_t bytes = (size_t)Nx * Ny * sizeof(double);
     double *f = nullptr;
     ENG_TRY(cudaMalloc((void **)&f, bytes), "autotune grid");
@@ -923,10 +925,7 @@ cj_status cj_autotune_engine(int Nx, int Ny, cj_stencil st, int *tile_rows, int 
     copies = std::min<long long>(copies, 256);
     copies = std::max<long long>(1, std::min<long long>(copies, (1LL << 24) / ((long long)Nx * Ny)));
     cj_status rc = CJ_OK;
-    for (int c = 0; c < 9 && rc == CJ_OK; ++c) {
-        // depth 4 of 5 and 9 points is timed from a shorter side of 512 on
-        if (dps[c] == 4 && st != CJ_ST17 && std::min(Nx, Ny) < kEngDeepMinSide) continue;
-        const long long cp = copies;
+    auto timed = [&](int ty, int depth, double *out) -> cj_status {
         Engine eng;
         Spec sp{};
         sp.Nx = Nx;
@@ -934,34 +933,67 @@ cj_status cj_autotune_engine(int Nx, int Ny, cj_stencil st, int *tile_rows, int 
         sp.st = st;
         sp.mode = CJ_FP32_INNER_DD;
         sp.inner_cycle = 0;
-        sp.depth = dps[c];
-        sp.ty = tys[c];
+        sp.depth = depth;
+        sp.ty = ty;
         sp.tol = 1e-15;
         sp.max_sweeps = 0;
-        rc = eng.init((int)cp, 1u << Engine::list_of(sp));
-        if (rc != CJ_OK) break;
-        std::vector<int> q(cp, -1);
-        for (long long k = 0; k < cp && rc == CJ_OK; ++k)
-            rc = eng.admit(sp, f, Nx, nullptr, 0, nullptr, 0, &q[k], true);  // results into own slot
+        cj_status rc = eng.init((int)copies, 1u << Engine::list_of(sp));
+        if (rc != CJ_OK) return rc;
+        std::vector<int> q(copies, -1);
+        auto admit_all = [&] {
+            cj_status rc = CJ_OK;
+            for (long long k = 0; k < copies && rc == CJ_OK; ++k)
+                rc = eng.admit(sp, f, Nx, nullptr, 0, nullptr, 0, &q[k], true);  // results into own slot
+            return rc;
+        };
+        rc = admit_all();
         if (rc == CJ_OK) rc = eng.run(2);  // capture and warm-up
-        if (rc != CJ_OK) break;
-        long long s0 = 0, s1 = 0;
-        for (long long k = 0; k < cp; ++k) s0 += eng.status(q[k]).sweeps;
+        // timed from the start again: at the deeper depths small problems end within a replay or two
+        for (long long k = 0; k < copies && rc == CJ_OK; ++k) rc = eng.release(q[k]);
+        if (rc == CJ_OK) rc = admit_all();
+        if (rc == CJ_OK) rc = eng.upload();
+        if (rc != CJ_OK) return rc;
+        long long sweeps = 0;
+        bool running = true;
         const auto t0 = Clock::now();
-        rc = eng.run(kReplays);
+        for (int rep = 0; rep < kReplays && running; ++rep) {
+            rc = eng.run(1);
+            if (rc != CJ_OK) return rc;
+            running = false;
+            for (long long k = 0; k < copies; ++k) running = running || eng.status(q[k]).phase != PHASE_RETIRED;
+        }
         const double secs = std::chrono::duration<double>(Clock::now() - t0).count();
-        if (rc != CJ_OK) break;
-        for (long long k = 0; k < cp; ++k) s1 += eng.status(q[k]).sweeps;
-        rate[c] = (double)Nx * Ny * (double)(s1 - s0) / secs / 1e9;
+        for (long long k = 0; k < copies; ++k) sweeps += eng.status(q[k]).sweeps;
+        *out = (double)Nx * Ny * (double)sweeps / secs / 1e9;
+        return CJ_OK;
+    };
+    for (int c = 0; c < 9 && rc == CJ_OK; ++c) {
+        if (dps[c] == 4 && st != CJ_ST17 && std::min(Nx, Ny) < kEngDeepMinSide) continue;
+        rc = timed(tys[c], dps[c], &rate[c]);
     }
-    cudaFree(f);
-    if (rc != CJ_OK) return rc;
     int best = 0;
     for (int c = 1; c < 9; ++c)
         if (rate[c] > rate[best]) best = c;
+    EngineTune choice{tys[best], dps[best]};
+    const int dflt = eng_default_depth(st);
+    if (std::find(dps, dps + 9, dflt) == dps + 9) {  // 17 points' is among the nine
+        double top = rate[best];
+        for (int k = 0; k < 2 && rc == CJ_OK; ++k) {
+            const int ty = k == 0 ? kEngTYDefault : tys[best];
+            if (k == 1 && ty == kEngTYDefault) break;
+            double v = 0.0;
+            rc = timed(ty, dflt, &v);
+            if (v > top) {
+                top = v;
+                choice = EngineTune{ty, dflt};
+            }
+        }
+    }
+    cudaFree(f);
+    if (rc != CJ_OK) return rc;
     {
         std::lock_guard<std::mutex> lk(g_engine_tune_mu);
-        g_engine_tune[stencil_slot(st)][size_class(Nx, Ny)] = EngineTune{tys[best], dps[best]};
+        g_engine_tune[stencil_slot(st)][size_class(Nx, Ny)] = choice;
     }
     if (tile_rows) *tile_rows = tys[best];
     if (depth) *depth = dps[best];

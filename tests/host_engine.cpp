@@ -194,10 +194,24 @@ void batch_while_tuned() {
     CHECK(!on_stream && live.empty());
 }
 
+// What the engine's autotuner records is what a batch of the class then runs, and no slower than what
+// an untuned one runs: the default depth where that is faster than those the tuner reports.
+void engine_tuned_depth() {
+    const cj_problem p = problem();
+    cj_result r{};
+    const double cases[3][5] = {{2000, 1000, 1000, 9000, 8}, {4000, 1000, 1000, 1000, 1}, {1000, 4000, 1000, 1000, 2}};
+    for (const double *c : cases) {
+        tune_engine(c[0], c[1], c[2], c[3]);
+        CHECK(cj_solve_batch(&p, 1, nullptr, &r) == CJ_OK);
+        CHECK(last_depth == (int)c[4]);
+    }
+}
+
 }  // namespace
 
 int main(int argc, char **argv) {
-    const std::map<std::string, void (*)()> scenarios{{"batch_while_tuned", batch_while_tuned}};
+    const std::map<std::string, void (*)()> scenarios{{"batch_while_tuned", batch_while_tuned},
+                                                          {"engine_tuned_depth", engine_tuned_depth}};
     const auto s = scenarios.find(argc > 1 ? argv[1] : "");
     if (s == scenarios.end()) return 2;
     s->second();
