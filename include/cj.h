@@ -326,12 +326,15 @@ cj_status cj_sweeps_f32(cj_plan *plan, const float *r, long long ld_r, float *e,
 cj_status cj_set_boundary(cj_plan *plan, const double *g, long long ld_g, void *stream);
 
 /*
- * cj_autotune_depth -- measure the FP32 sweep at temporal depths 1, 2, 4 and 8 on an Nx x Ny
- * grid (`sweeps` >= 8 sweeps each, CUDA events on `stream`), and record the fastest for the
- * stencil and size class (grids whose node counts are within a factor 4 share a class) in a
- * per-process table; FP32-inner plans created afterwards with temporal_depth = 0 use it.
- * *best_depth (may be NULL) receives the winner, gupd[4] (may be NULL) the measured
- * grid-point updates per second (1e9) at depths 1, 2, 4, 8.  Allocates a temporary plan.
+ * cj_autotune_depth -- measure the FP32 sweep at temporal depths 1, 2, 4 and 8 and at the plan's own
+ * (cj_options' 0) on an Nx x Ny grid (`sweeps` >= 8 sweeps each, CUDA events on `stream`), and
+ * record the fastest for the stencil and size class (grids whose node counts are within a factor 4
+ * share a class) in a per-process table; FP32-inner plans created afterwards with
+ * temporal_depth = 0 use it.
+ * *best_depth (may be NULL) receives the fastest of depths 1, 2, 4 and 8, which is the recorded
+ * choice unless the plan's own depth was faster still (such a class stays as if not tuned), gupd[4]
+ * (may be NULL) the measured grid-point updates per second (1e9) at depths 1, 2, 4, 8.  Allocates
+ * a temporary plan.
  */
 cj_status cj_autotune_depth(int Nx, int Ny, cj_stencil st, int sweeps, void *stream, int *best_depth,
                             double *gupd);

@@ -381,8 +381,8 @@ def cj_set_boundary(plan, g, stream=None) -> None:
 
 
 def cj_autotune_depth(Nx: int, Ny: int, st: int, sweeps: int = 64, stream=None) -> dict:
-    """Time FP32 sweeps at temporal depths 1, 2, 4, 8 and record the fastest for this
-    stencil and size class; returns {"best": depth, "gupd": {depth: rate}}."""
+    """Time FP32 sweeps at temporal depths 1, 2, 4, 8 and the plan's own and record the fastest for
+    this stencil and size class; returns the four as {"best": depth, "gupd": {depth: rate}}."""
     best = ctypes.c_int()
     rates = (ctypes.c_double * 4)()
     rc = _lib().cj_autotune_depth(Nx, Ny, st, sweeps, _stream(stream), ctypes.byref(best), rates)

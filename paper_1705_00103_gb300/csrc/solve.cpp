@@ -30,7 +30,7 @@ namespace {
 thread_local char g_err[256] = "";
 
 // Autotuned FP32 temporal depth per (stencil, size class); size class = floor(log2(Nx*Ny)/2),
-// i.e. grids within a factor 2 of each other per side share a class.  0 = not tuned.
+// i.e. grids within a factor 2 of each other per side share a class.  0 = the plan's own depth.
 std::mutex g_tune_mu;
 int g_tuned_depth[3][32] = {};
 
@@ -973,17 +973,19 @@ cj_status cj_autotune_depth(int Nx, int Ny, cj_stencil st, int sweeps, void *str
     if (Nx < 1 || Ny < 1 || sweeps < 8) return CJ_ERR_INVALID_ARG;
     if (st != CJ_ST5 && st != CJ_ST9 && st != CJ_ST17) return CJ_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
-    const int depths[4] = {1, 2, 4, 8};
-    double rate[4] = {0, 0, 0, 0};
-    int best = 1;
+    // the four reported depths, and the plan's own (rtile.cu) where it is not one of them
+    const int own = rtile_depth(st, Nx, Ny, 64);
+    const int depths[5] = {1, 2, 4, 8, own};
+    const int n = std::find(depths, depths + 4, own) == depths + 4 ? 5 : 4;
+    double rate[5] = {0, 0, 0, 0, 0};
     cudaEvent_t e0, e1;
     CJ_TRY(cudaEventCreate(&e0), "autotune event");
     CJ_TRY(cudaEventCreate(&e1), "autotune event");
-    for (int k = 0; k < 4; ++k) {
+    for (int k = 0; k < n; ++k) {
         cj_options o{};
         o.precision = CJ_FP32_INNER;
         o.inner_cycle = 64;
-        o.temporal_depth = depths[k];
+        o.temporal_depth = 1;
         cj_plan *p = nullptr;
         cj_status st2 = cj_plan_create(Nx, Ny, st, CJ_BC_DIRICHLET0, 1e-6, &o, &p);
         if (st2 != CJ_OK) {
@@ -991,11 +993,13 @@ cj_status cj_autotune_depth(int Nx, int Ny, cj_stencil st, int sweeps, void *str
             cudaEventDestroy(e1);
             return st2;
         }
+        p->depth = depths[k];
         float *cur = p->e0, *nxt = p->e1;
         long long launches = 0;
-        cudaError_t err = fp32_sweeps(p, &cur, &nxt, p->rt, 0, 8, s, &launches);  // warm-up
+        const long long count = k < 4 ? sweeps : (sweeps + own - 1LL) / own * own;  // whole launches of the own depth
+        cudaError_t err = fp32_sweeps(p, &cur, &nxt, p->rt, 0, depths[k] > 8 ? depths[k] : 8, s, &launches);  // warm-up
         if (err == cudaSuccess) err = cudaEventRecord(e0, s);
-        if (err == cudaSuccess) err = fp32_sweeps(p, &cur, &nxt, p->rt, 0, sweeps, s, &launches);
+        if (err == cudaSuccess) err = fp32_sweeps(p, &cur, &nxt, p->rt, 0, count, s, &launches);
         if (err == cudaSuccess) err = cudaEventRecord(e1, s);
         if (err == cudaSuccess) err = cudaEventSynchronize(e1);
         float ms = 0.0f;
@@ -1007,19 +1011,19 @@ cj_status cj_autotune_depth(int Nx, int Ny, cj_stencil st, int sweeps, void *str
             cudaEventDestroy(e1);
             return CJ_ERR_CUDA;
         }
-        rate[k] = (double)Nx * Ny * sweeps / (ms * 1e-3) / 1e9;
+        rate[k] = (double)Nx * Ny * count / (ms * 1e-3) / 1e9;
     }
     int kbest = 0;  // the fastest depth; the shallower one on a tie
     for (int k = 1; k < 4; ++k)
         if (rate[k] > rate[kbest]) kbest = k;
-    best = depths[kbest];
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
-        g_tuned_depth[stencil_slot(st)][size_class(Nx, Ny)] = best;
+        // (0: the plan's own depth at each size)
+        g_tuned_depth[stencil_slot(st)][size_class(Nx, Ny)] = rate[4] > rate[kbest] ? 0 : depths[kbest];
     }
-    if (best_depth) *best_depth = best;
+    if (best_depth) *best_depth = depths[kbest];
     if (gupd)
         for (int k = 0; k < 4; ++k) gupd[k] = rate[k];
     return CJ_OK;

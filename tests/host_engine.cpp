@@ -151,6 +151,20 @@ cudaError_t eng_launch_import(const EngineDev &e, int slot, int, const double *,
     e.slots[slot].phase = PHASE_OUTER;
     return cudaSuccess;
 }
+cudaError_t launch_sweep32(const cj_plan *, const float *, const float *, float *, float, cudaStream_t) {
+    return last_depth = 1, clock_us += launch_us[1], cudaSuccess;
+}
+cudaError_t launch_sweep32_rtile(const cj_plan *, const float *, const float *, float *, const float *, int k,
+                                 cudaStream_t) {
+    return last_depth = k, clock_us += launch_us[k], cudaSuccess;
+}
+cudaError_t launch_import32(const cj_plan *, const float *, long long, float *, cudaStream_t) { return cudaSuccess; }
+cudaError_t launch_export32(const cj_plan *, const float *, float *, long long, cudaStream_t) { return cudaSuccess; }
+int cluster_solve_size(const cj_plan *) { return 0; }
+cudaError_t rtile_prepare(int) { return cudaSuccess; }
+int rtile_depth(int, int, int, long long sweeps) { return sweeps < 12 ? (int)sweeps : 12; }
+March plan_march(int, int Ny, int, bool) { return March{1, 1, Ny}; }
+Sweep64Shape sweep64_shape(int, int Ny, int) { return Sweep64Shape{Ny, 1, 1}; }
 cudaError_t eng_prepare() { return cudaSuccess; }
 int eng_default_depth(int st) { return st == 17 ? 4 : 8; }
 int eng_list(int st, int Nx, int Ny) { return 2 * stencil_slot(st) + ((long long)Nx * Ny > (1LL << 20) ? 1 : 0); }
@@ -207,11 +221,32 @@ void engine_tuned_depth() {
     }
 }
 
+// cj_autotune_depth leaves a class at the plan's own depth where that is faster than the four it reports.
+void plan_tuned_depth() {
+    for (const double own : {4.0, 12.0}) {  // us of a launch of 12 sweeps; one of k of the four: 2 + k / 2
+        for (int k = 1; k <= kRtMaxDepth; ++k) launch_us[k] = k == 12 ? own : 2.0 + 0.5 * k;
+        int best = 0;
+        double gupd[4];
+        CHECK(cj_autotune_depth(N, N, CJ_ST9, 8, nullptr, &best, gupd) == CJ_OK);
+        CHECK(best == 8 && gupd[3] > gupd[2] && gupd[2] > gupd[1] && gupd[1] > gupd[0]);
+        cj_options o{};
+        o.precision = CJ_FP32_INNER;
+        o.inner_cycle = 64;
+        cj_plan *p = nullptr;
+        CHECK(cj_plan_create(N, N, CJ_ST9, CJ_BC_DIRICHLET0, 1e-6, &o, &p) == CJ_OK);
+        static float r[N * N], e[N * N];
+        CHECK(cj_sweeps_f32(p, r, N, e, N, 0, 24, nullptr) == CJ_OK);
+        CHECK(last_depth == (own == 4.0 ? 12 : 8));
+        cj_plan_destroy(p);
+    }
+}
+
 }  // namespace
 
 int main(int argc, char **argv) {
     const std::map<std::string, void (*)()> scenarios{{"batch_while_tuned", batch_while_tuned},
-                                                          {"engine_tuned_depth", engine_tuned_depth}};
+                                                          {"engine_tuned_depth", engine_tuned_depth},
+                                                          {"plan_tuned_depth", plan_tuned_depth}};
     const auto s = scenarios.find(argc > 1 ? argv[1] : "");
     if (s == scenarios.end()) return 2;
     s->second();
