@@ -19,11 +19,12 @@
 namespace {
 
 // Sweep launches per captured graph: a replay advances a slot by up to 256 sweeps (8 per launch; 17
-// points: 128).  They are one engine step, or kShortSteps where every inner cycle at hand ends
-// within fewer launches than that: a step's five other kernels cost about 20 us, against 10 us a
-// launch (measured, steps of 8 launches -> 32: 32 problems of 64 .. 1024 a side 17.3 -> 16.4 ms, 8 served
-// requests of 32 .. 300 4.7 -> 4.2 ms), but a slot waits for its step's end once its cycle has ended
-// (16 problems of 8 .. 24 a side, cycles of 4 to 8 launches: 1.84 ms with 8, 2.03 with 32).
+// points: 128).  They are one engine step, or kShortSteps where the inner cycle of every slot in use
+// ends within fewer launches than that (a graph of each kind, captured when it is first needed): a
+// step's five other kernels cost about 20 us, against 10 us a launch (measured, steps of 8 launches ->
+// 32: 32 problems of 64 .. 1024 a side 17.3 -> 16.4 ms, 8 served requests of 32 .. 300 4.7 -> 4.2 ms),
+// but a slot waits for its step's end once its cycle has ended (16 problems of 8 .. 24 a side, cycles
+// of 4 to 8 launches: 1.84 ms with 8, 2.03 with 32; one served request of 11^2 0.46 and 0.59 ms).
 constexpr int kSweepsPerGraph = 32, kShortSteps = 4;
 // Shorter side from which the autotuner times and reports depth 4 of 5 and 9 points (the default depth
 // is timed at every size).
@@ -134,8 +135,7 @@ class Engine {
         cudaStreamSynchronize(s_);
         for (int q = 0; q < max_slots_; ++q)
             if (mem_[q].base) cudaFree(mem_[q].base);
-        if (gexec_) cudaGraphExecDestroy(gexec_);
-        if (graph_) cudaGraphDestroy(graph_);
+        drop_graphs();
         cudaFree(d_.slots);
         cudaFree(d_.status);
         cudaFree(d_.ntiles);
@@ -302,15 +302,16 @@ class Engine {
     cj_status run(int replays) {
         cj_status st = upload();
         if (st != CJ_OK) return st;
-        if (!gexec_) {
-            st = capture();
+        StepGraph &G = graphs_[steps_per_graph_ == kShortSteps];
+        if (!G.exec) {
+            st = capture(G);
             if (st != CJ_OK) return st;
         }
-        if (tile_grid_ && grids_dirty_) {
-            st = set_tile_grid();
+        if (tile_grid_ && G.grids_dirty) {
+            st = set_tile_grid(G);
             if (st != CJ_OK) return st;
         }
-        for (int k = 0; k < replays; ++k) ENG_TRY(cudaGraphLaunch(gexec_, s_), "graph launch");
+        for (int k = 0; k < replays; ++k) ENG_TRY(cudaGraphLaunch(G.exec, s_), "graph launch");
         int nlists = 0;
         for (int l = 0; l < kEngBranches; ++l) nlists += (int)(lists_ >> l & 1u);
         launches_ += (long long)replays * (steps_per_graph_ * 5 + nlists * kSweepsPerGraph);
@@ -326,6 +327,29 @@ class Engine {
     int steps_per_graph() const { return steps_per_graph_; }
 
   private:
+    // a kernel node whose grid follows the tile list (list -1) or a sweep list; blocks it launches
+    // in the instantiated graph (0: those of the capture)
+    struct GridNode {
+        cudaGraphNode_t node;
+        int list, blocks;
+    };
+
+    // A captured graph of steps.
+    struct StepGraph {
+        cudaGraph_t graph = nullptr;
+        cudaGraphExec_t exec = nullptr;
+        std::vector<GridNode> nodes;
+        bool grids_dirty = true;
+    };
+
+    void drop_graphs() {
+        for (StepGraph &G : graphs_) {
+            if (G.exec) cudaGraphExecDestroy(G.exec);
+            if (G.graph) cudaGraphDestroy(G.graph);
+            G = StepGraph{};
+        }
+    }
+
     cj_status ensure_tile_capacity(int n) {
         if (n <= tile_cap_) return CJ_OK;
         int cap = std::max(n, 2 * tile_cap_);
@@ -334,12 +358,7 @@ class Engine {
         cudaFree(d_.tiles);
         d_.tiles = t;
         tile_cap_ = cap;
-        if (gexec_) {  // the graph bakes the table pointer in: capture again
-            cudaGraphExecDestroy(gexec_);
-            gexec_ = nullptr;
-            cudaGraphDestroy(graph_);
-            graph_ = nullptr;
-        }
+        drop_graphs();  // the graphs bake the table pointer in: capture again
         return CJ_OK;
     }
 
@@ -372,7 +391,11 @@ class Engine {
                 "item offsets");
         ENG_TRY(cudaStreamSynchronize(s_), "tile sync");
         tiles_dirty_ = false;
-        grids_dirty_ = true;
+        for (StepGraph &G : graphs_) G.grids_dirty = true;
+        long long cycle = 0;  // launches of the longest inner cycle
+        for (int q = 0; q < max_slots_; ++q)
+            if (used_[q]) cycle = std::max(cycle, host_[q].M_in / host_[q].depth);
+        steps_per_graph_ = cycle >= kSweepsPerGraph ? 1 : kShortSteps;
         return CJ_OK;
     }
 
@@ -384,20 +407,11 @@ class Engine {
         cudaFree(d_.items);
         d_.items = t;
         item_cap_ = cap;
-        if (gexec_) {  // the graph bakes the table pointer in: capture again
-            cudaGraphExecDestroy(gexec_);
-            gexec_ = nullptr;
-            cudaGraphDestroy(graph_);
-            graph_ = nullptr;
-        }
+        drop_graphs();  // the graphs bake the table pointer in: capture again
         return CJ_OK;
     }
 
-    cj_status capture() {
-        long long cycle = 0;  // launches of the longest inner cycle
-        for (int q = 0; q < max_slots_; ++q)
-            if (used_[q]) cycle = std::max(cycle, host_[q].M_in / host_[q].depth);
-        steps_per_graph_ = cycle >= kSweepsPerGraph ? 1 : kShortSteps;
+    cj_status capture(StepGraph &G) {
         cudaGraph_t g = nullptr;
         ENG_TRY(cudaStreamBeginCapture(s_, cudaStreamCaptureModeThreadLocal), "begin capture");
         cudaError_t err = cudaSuccess;
@@ -406,9 +420,9 @@ class Engine {
                                   s_);
         cudaError_t e2 = cudaStreamEndCapture(s_, &g);
         if (err == cudaSuccess) err = e2;
-        if (err == cudaSuccess) err = cudaGraphInstantiate(&gexec_, g, 0);
-        tile_nodes_.clear();
-        grids_dirty_ = true;
+        if (err == cudaSuccess) err = cudaGraphInstantiate(&G.exec, g, 0);
+        G.nodes.clear();
+        G.grids_dirty = true;
         if (err == cudaSuccess && tile_grid_) {  // the nodes whose grid follows the tile list
             size_t n = 0;
             err = cudaGraphGetNodes(g, nullptr, &n);
@@ -422,11 +436,11 @@ class Engine {
                 err = cudaGraphKernelNodeGetParams(nodes[k], &kp);
                 const int list = err == cudaSuccess ? eng_list_of_kernel(kp.func) : -1;
                 if (err == cudaSuccess && (list >= 0 || eng_is_tile_kernel(kp.func)))
-                    tile_nodes_.push_back({nodes[k], list, 0});
+                    G.nodes.push_back({nodes[k], list, 0});
             }
         }
         if (err == cudaSuccess) {
-            graph_ = g;  // kept: the tile kernels' nodes are updated through it
+            G.graph = g;  // kept: the tile kernels' nodes are updated through it
         } else if (g) {
             cudaGraphDestroy(g);
         }
@@ -436,26 +450,19 @@ class Engine {
 
     // The tile kernels of the instantiated graph launch one block per tile, the sweep kernels one per
     // item of their list, from now on.
-    cj_status set_tile_grid() {
-        for (GridNode &n : tile_nodes_) {
+    cj_status set_tile_grid(StepGraph &G) {
+        for (GridNode &n : G.nodes) {
             const int want = std::max(1, n.list < 0 ? *h_ntiles_ : h_off_[n.list + 1] - h_off_[n.list]);
             if (want == n.blocks) continue;
             cudaKernelNodeParams kp{};
             ENG_TRY(cudaGraphKernelNodeGetParams(n.node, &kp), "tile node params");
             kp.gridDim = dim3((unsigned)want);
-            ENG_TRY(cudaGraphExecKernelNodeSetParams(gexec_, n.node, &kp), "tile grid update");
+            ENG_TRY(cudaGraphExecKernelNodeSetParams(G.exec, n.node, &kp), "tile grid update");
             n.blocks = want;
         }
-        grids_dirty_ = false;
+        G.grids_dirty = false;
         return CJ_OK;
     }
-
-    // a kernel node whose grid follows the tile list (list -1) or a sweep list; blocks it launches
-    // in the instantiated graph (0: those of the capture)
-    struct GridNode {
-        cudaGraphNode_t node;
-        int list, blocks;
-    };
 
     int dev_ = 0, max_slots_ = 0, grid_tiles_ = 0, grid_slots_ = 0, rt_blocks_ = 0;
     unsigned lists_ = 0;
@@ -475,10 +482,8 @@ class Engine {
     bool tiles_dirty_ = true;
     SlotStatus *h_status_ = nullptr;
     int *h_ntiles_ = nullptr;
-    cudaGraphExec_t gexec_ = nullptr;
-    cudaGraph_t graph_ = nullptr;
-    bool tile_grid_ = false, grids_dirty_ = true;
-    std::vector<GridNode> tile_nodes_;
+    StepGraph graphs_[2];  // of one step, of kShortSteps
+    bool tile_grid_ = false;
     long long launches_ = 0;
 };
 

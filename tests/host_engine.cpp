@@ -22,6 +22,7 @@ bool retire = true;                            // a graph replay ends every slot
 double sweeps_per_replay[kRtMaxDepth + 1];     // by depth, where it does not end them
 double clock_us = 0.0, launch_us[kRtMaxDepth + 1];
 int last_depth = 0;                            // of the last FP32 sweep launch, or imported slot
+std::atomic<int> last_steps{0}, instances{0};  // engine steps of the last replay, graphs instantiated
 
 struct Step {
     EngineDev e;
@@ -111,6 +112,7 @@ cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t *g) {
     return cudaSuccess;
 }
 cudaError_t cudaGraphInstantiate(cudaGraphExec_t *x, cudaGraph_t g, unsigned long long) {
+    ++instances;
     return *x = (cudaGraphExec_t) new Steps(*(Steps *)g), cudaSuccess;
 }
 cudaError_t cudaGraphDestroy(cudaGraph_t g) { return delete (Steps *)g, cudaSuccess; }
@@ -124,6 +126,7 @@ cudaError_t cudaGraphExecKernelNodeSetParams(cudaGraphExec_t, cudaGraphNode_t, c
 cudaError_t cudaGraphLaunch(cudaGraphExec_t x, cudaStream_t) {
     std::this_thread::sleep_for(std::chrono::microseconds(200));  // the engine's autotuner reads the wall clock
     const Steps &steps = *(Steps *)x;
+    last_steps = (int)steps.size();
     const EngineDev &e = steps[0].e;
     for (int q = 0; q < e.max_slots; ++q) {
         SlotDev &S = e.slots[q];
@@ -241,12 +244,38 @@ void plan_tuned_depth() {
     }
 }
 
+void serve(cj_server *sv, int n) {
+    static double f[300 * 300], u[300 * 300];
+    uint64_t t = 0;
+    CHECK(cj_submit(sv, n, n, CJ_ST9, 1e-6, f, &t) == CJ_OK);
+    cj_status st = CJ_PENDING;
+    while (st == CJ_PENDING) st = cj_poll(sv, t, u, nullptr);
+    CHECK(st == CJ_OK);
+}
+
+// A request's steps are those of the requests beside it, whatever a lane ran before: one step of 32
+// sweep launches for long inner cycles, four of 8 for short ones.
+void steps_follow_requests() {
+    for (const bool large_first : {true, false}) {
+        cj_server *sv = nullptr;
+        CHECK(cj_server_create(1 << 30, 4, &sv) == CJ_OK);
+        for (int k = 0; k < 4; ++k) {
+            const bool large = (k % 2 == 0) == large_first;
+            serve(sv, large ? 300 : 16);
+            CHECK(last_steps == (large ? 1 : 4));
+        }
+        cj_server_destroy(sv);
+        CHECK(live.empty());
+    }
+}
+
 }  // namespace
 
 int main(int argc, char **argv) {
     const std::map<std::string, void (*)()> scenarios{{"batch_while_tuned", batch_while_tuned},
                                                           {"engine_tuned_depth", engine_tuned_depth},
-                                                          {"plan_tuned_depth", plan_tuned_depth}};
+                                                          {"plan_tuned_depth", plan_tuned_depth},
+                                                          {"steps_follow_requests", steps_follow_requests}};
     const auto s = scenarios.find(argc > 1 ? argv[1] : "");
     if (s == scenarios.end()) return 2;
     s->second();

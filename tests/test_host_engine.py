@@ -19,7 +19,8 @@ def program(tmp_path_factory):
     return exe
 
 
-@pytest.mark.parametrize("scenario", ["batch_while_tuned", "engine_tuned_depth", "plan_tuned_depth"])
+@pytest.mark.parametrize("scenario", ["batch_while_tuned", "engine_tuned_depth", "plan_tuned_depth",
+                                      "steps_follow_requests"])
 def test_scenario(program, scenario):
     r = subprocess.run([program, scenario], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stdout + r.stderr
