@@ -126,7 +126,10 @@ class Engine {
         ENG_TRY(cudaMallocHost(&h_status_, sizeof(SlotStatus) * max_slots), "engine status (host)");
         ENG_TRY(cudaMallocHost(&h_ntiles_, sizeof(int)), "engine tile count (host)");
         ENG_TRY(cudaMallocHost(&h_off_, sizeof(int) * (kEngLists + 1)), "engine item offsets (host)");
-        return ensure_tile_capacity(1024);
+        // room for the tables of a lane's ordinary load: each growth is an allocation, and captures the
+        // graphs again
+        const cj_status st = ensure_item_capacity(4096);
+        return st != CJ_OK ? st : ensure_tile_capacity(1024);
     }
 
     void destroy() {

@@ -245,7 +245,7 @@ void plan_tuned_depth() {
 }
 
 void serve(cj_server *sv, int n) {
-    static double f[300 * 300], u[300 * 300];
+    static double f[1000 * 1000], u[1000 * 1000];
     uint64_t t = 0;
     CHECK(cj_submit(sv, n, n, CJ_ST9, 1e-6, f, &t) == CJ_OK);
     cj_status st = CJ_PENDING;
@@ -269,13 +269,23 @@ void steps_follow_requests() {
     }
 }
 
+// A fresh server's graph is not captured again for each larger request of its first ones.
+void graph_kept_in_first_burst() {
+    cj_server *sv = nullptr;
+    CHECK(cj_server_create(1 << 30, 4, &sv) == CJ_OK);
+    for (const int n : {200, 300, 600, 1000}) serve(sv, n);
+    CHECK(instances == 1);
+    cj_server_destroy(sv);
+}
+
 }  // namespace
 
 int main(int argc, char **argv) {
     const std::map<std::string, void (*)()> scenarios{{"batch_while_tuned", batch_while_tuned},
                                                           {"engine_tuned_depth", engine_tuned_depth},
                                                           {"plan_tuned_depth", plan_tuned_depth},
-                                                          {"steps_follow_requests", steps_follow_requests}};
+                                                          {"steps_follow_requests", steps_follow_requests},
+                                                          {"graph_kept_in_first_burst", graph_kept_in_first_burst}};
     const auto s = scenarios.find(argc > 1 ? argv[1] : "");
     if (s == scenarios.end()) return 2;
     s->second();

@@ -20,7 +20,7 @@ def program(tmp_path_factory):
 
 
 @pytest.mark.parametrize("scenario", ["batch_while_tuned", "engine_tuned_depth", "plan_tuned_depth",
-                                      "steps_follow_requests"])
+                                      "steps_follow_requests", "graph_kept_in_first_burst"])
 def test_scenario(program, scenario):
     r = subprocess.run([program, scenario], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stdout + r.stderr
