@@ -18,14 +18,16 @@
 
 namespace {
 
-// Sweep launches per captured graph: a replay advances a slot by up to 256 sweeps (8 per launch; 17
-// points: 128).  They are one engine step, or kShortSteps where the inner cycle of every slot in use
-// ends within fewer launches than that (a graph of each kind, captured when it is first needed): a
-// step's five other kernels cost about 20 us, against 10 us a launch (measured, steps of 8 launches ->
-// 32: 32 problems of 64 .. 1024 a side 17.3 -> 16.4 ms, 8 served requests of 32 .. 300 4.7 -> 4.2 ms),
-// but a slot waits for its step's end once its cycle has ended (16 problems of 8 .. 24 a side, cycles
-// of 4 to 8 launches: 1.84 ms with 8, 2.03 with 32; one served request of 11^2 0.46 and 0.59 ms).
-constexpr int kSweepsPerGraph = 32, kShortSteps = 4;
+// Sweep launches of an engine step, which is what a captured graph holds: the first of these that the
+// longest inner cycle of the slots in use ends within, or the last (8 sweeps per launch, so a replay of
+// that advances a slot by up to 256; 17 points: 128).  One graph of each kind, captured when it is first
+// needed.  A step's five other kernels cost about 20 us, against 10 us a launch (steps of 8 launches ->
+// 32: 32 problems of 64 .. 1024 a side 17.3 -> 16.4 ms, 8 served requests of 32 .. 300 4.7 -> 4.2 ms), but a
+// slot waits for its step's end once its cycle has ended, and a request for the replay's (cycles of 4 to 8
+// launches, steps of 32 launches / replays of four steps of 8 / steps of 8: 16 problems of 8 .. 24 a side
+// in a batch 2.03 / 1.80 / 1.64 ms, as served requests together 1.87 / 1.95 / 1.72, one request 0.58 / 0.46 /
+// 0.46; cycles of 16, replays of four steps of 8 / steps of 16: 24 problems of 64^2 2.49 / 2.38).
+constexpr int kStepKinds = 3, kStepLaunches[kStepKinds] = {8, 16, 32};
 // Shorter side from which the autotuner times and reports depth 4 of 5 and 9 points (the default depth
 // is timed at every size).
 constexpr int kEngDeepMinSide = 512;
@@ -305,7 +307,7 @@ class Engine {
     cj_status run(int replays) {
         cj_status st = upload();
         if (st != CJ_OK) return st;
-        StepGraph &G = graphs_[steps_per_graph_ == kShortSteps];
+        StepGraph &G = graphs_[kind_];
         if (!G.exec) {
             st = capture(G);
             if (st != CJ_OK) return st;
@@ -317,7 +319,7 @@ class Engine {
         for (int k = 0; k < replays; ++k) ENG_TRY(cudaGraphLaunch(G.exec, s_), "graph launch");
         int nlists = 0;
         for (int l = 0; l < kEngBranches; ++l) nlists += (int)(lists_ >> l & 1u);
-        launches_ += (long long)replays * (steps_per_graph_ * 5 + nlists * kSweepsPerGraph);
+        launches_ += (long long)replays * (5 + nlists * kStepLaunches[kind_]);
         ENG_TRY(cudaMemcpyAsync(h_status_, d_.status, sizeof(SlotStatus) * max_slots_,
                                 cudaMemcpyDeviceToHost, s_), "status readback");
         ENG_TRY(cudaStreamSynchronize(s_), "step sync");
@@ -327,7 +329,6 @@ class Engine {
     const SlotStatus &status(int q) const { return h_status_[q]; }
     bool used(int q) const { return used_[q] != 0; }
     long long launches() const { return launches_; }
-    int steps_per_graph() const { return steps_per_graph_; }
 
   private:
     // a kernel node whose grid follows the tile list (list -1) or a sweep list; blocks it launches
@@ -337,7 +338,7 @@ class Engine {
         int list, blocks;
     };
 
-    // A captured graph of steps.
+    // A captured step.
     struct StepGraph {
         cudaGraph_t graph = nullptr;
         cudaGraphExec_t exec = nullptr;
@@ -397,8 +398,9 @@ class Engine {
         for (StepGraph &G : graphs_) G.grids_dirty = true;
         long long cycle = 0;  // launches of the longest inner cycle
         for (int q = 0; q < max_slots_; ++q)
-            if (used_[q]) cycle = std::max(cycle, host_[q].M_in / host_[q].depth);
-        steps_per_graph_ = cycle >= kSweepsPerGraph ? 1 : kShortSteps;
+            if (used_[q]) cycle = std::max(cycle, (host_[q].M_in + host_[q].depth - 1) / host_[q].depth);
+        kind_ = 0;
+        while (kind_ < kStepKinds - 1 && kStepLaunches[kind_] < cycle) ++kind_;
         return CJ_OK;
     }
 
@@ -417,10 +419,8 @@ class Engine {
     cj_status capture(StepGraph &G) {
         cudaGraph_t g = nullptr;
         ENG_TRY(cudaStreamBeginCapture(s_, cudaStreamCaptureModeThreadLocal), "begin capture");
-        cudaError_t err = cudaSuccess;
-        for (int k = 0; k < steps_per_graph_ && err == cudaSuccess; ++k)
-            err = eng_launch_step(d_, grid_tiles_, grid_slots_, lists_, rt_blocks_, br_, kSweepsPerGraph / steps_per_graph_,
-                                  s_);
+        cudaError_t err =
+            eng_launch_step(d_, grid_tiles_, grid_slots_, lists_, rt_blocks_, br_, kStepLaunches[kind_], s_);
         cudaError_t e2 = cudaStreamEndCapture(s_, &g);
         if (err == cudaSuccess) err = e2;
         if (err == cudaSuccess) err = cudaGraphInstantiate(&G.exec, g, 0);
@@ -469,7 +469,7 @@ class Engine {
 
     int dev_ = 0, max_slots_ = 0, grid_tiles_ = 0, grid_slots_ = 0, rt_blocks_ = 0;
     unsigned lists_ = 0;
-    int steps_per_graph_ = 1;
+    int kind_ = 0;  // of the step for the slots in use
     EngineBranches br_;
     cudaStream_t s_ = nullptr;
     EngineDev d_{};
@@ -485,7 +485,7 @@ class Engine {
     bool tiles_dirty_ = true;
     SlotStatus *h_status_ = nullptr;
     int *h_ntiles_ = nullptr;
-    StepGraph graphs_[2];  // of one step, of kShortSteps
+    StepGraph graphs_[kStepKinds];
     bool tile_grid_ = false;
     long long launches_ = 0;
 };
@@ -746,7 +746,7 @@ struct cj_server {
             std::vector<std::pair<int, uint64_t>> done;
             {
                 std::lock_guard<std::mutex> lk(mu);
-                steps += L.eng.steps_per_graph();
+                steps += 1;
                 for (auto &kv : L.by_slot)
                     if (L.eng.status(kv.first).phase == PHASE_RETIRED) done.push_back(kv);
             }
@@ -870,8 +870,8 @@ cj_status cj_solve_batch(const cj_problem *problems, int n, void *stream, cj_res
         const long long outer = max_sweeps / M_in + 1;
         max_steps = std::max(max_steps, outer * (M_in / sp.depth + 2) + 4);
     }
-    // every slot retires within max_steps engine steps (its outer-step budget)
-    const long long max_replays = max_steps / eng.steps_per_graph() + 2;
+    // every slot retires within max_steps engine steps (its outer-step budget), one a replay
+    const long long max_replays = max_steps + 2;
     bool all = false;
     for (long long rep = 0; rep < max_replays && !all; ++rep) {
         st = eng.run(1);

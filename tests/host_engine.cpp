@@ -22,7 +22,7 @@ bool retire = true;                            // a graph replay ends every slot
 double sweeps_per_replay[kRtMaxDepth + 1];     // by depth, where it does not end them
 double clock_us = 0.0, launch_us[kRtMaxDepth + 1];
 int last_depth = 0;                            // of the last FP32 sweep launch, or imported slot
-std::atomic<int> last_steps{0}, instances{0};  // engine steps of the last replay, graphs instantiated
+std::atomic<int> last_step{0}, instances{0};   // sweep launches of the last replay, graphs instantiated
 
 struct Step {
     EngineDev e;
@@ -126,7 +126,8 @@ cudaError_t cudaGraphExecKernelNodeSetParams(cudaGraphExec_t, cudaGraphNode_t, c
 cudaError_t cudaGraphLaunch(cudaGraphExec_t x, cudaStream_t) {
     std::this_thread::sleep_for(std::chrono::microseconds(200));  // the engine's autotuner reads the wall clock
     const Steps &steps = *(Steps *)x;
-    last_steps = (int)steps.size();
+    last_step = 0;
+    for (const Step &t : steps) last_step += t.sweeps;
     const EngineDev &e = steps[0].e;
     for (int q = 0; q < e.max_slots; ++q) {
         SlotDev &S = e.slots[q];
@@ -253,8 +254,8 @@ void serve(cj_server *sv, int n) {
     CHECK(st == CJ_OK);
 }
 
-// A request's steps are those of the requests beside it, whatever a lane ran before: one step of 32
-// sweep launches for long inner cycles, four of 8 for short ones.
+// A request's steps are those of the requests beside it, whatever a lane ran before: 32 sweep launches
+// for long inner cycles, 8 for the shortest.
 void steps_follow_requests() {
     for (const bool large_first : {true, false}) {
         cj_server *sv = nullptr;
@@ -262,7 +263,7 @@ void steps_follow_requests() {
         for (int k = 0; k < 4; ++k) {
             const bool large = (k % 2 == 0) == large_first;
             serve(sv, large ? 300 : 16);
-            CHECK(last_steps == (large ? 1 : 4));
+            CHECK(last_step == (large ? 32 : 8));
         }
         cj_server_destroy(sv);
         CHECK(live.empty());
