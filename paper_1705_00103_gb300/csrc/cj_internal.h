@@ -140,7 +140,16 @@ bool cluster_solve_pays(const cj_plan *p);
 // res_dev[0..5] = status, sweeps, cycles, rho, rinf, fl
 cudaError_t launch_cluster_solve(const cj_plan *p, double *res_dev, cudaStream_t s);
 
-// ---- the FP64 sweep (sweep64.cu); its launches may overlap the end of the one before in the stream
+// ---- Programmatic dependent launch, which the launches of sweeps (sweep64.cu, rtile.cu, ff.cu, the
+// engine's lists) ask for: a grid may begin while the one before it in the stream (or graph) ends, and
+// its threads run griddepcontrol.wait, which returns once that grid has completed and its writes are
+// visible.  Every thread waits before it ends and before it lets its dependents begin, so one grid's
+// completion implies that of all before it.  What is read or written after the wait is as after an
+// ordinary launch, through any cache.  Before the wait a grid may read only what the grid right
+// before it does not write: the weights and positions of a table, and the right-hand side r of an FP32
+// sweep.
+
+// ---- the FP64 sweep (sweep64.cu)
 Sweep64Shape sweep64_shape(int Nx, int Ny, int st);
 cudaError_t launch_sweep64(const cj_plan *p, const double *u, double *out, double w,
                            cudaStream_t s);
@@ -184,7 +193,8 @@ cudaError_t launch_defect_dd64(const cj_plan *p, const double *uh, const double 
                                double *e_zero, cudaStream_t s);
 cudaError_t launch_correct_dd64(const cj_plan *p, double *uh, double *ul, const double *e,
                                 cudaStream_t s);
-// register-tile FP32 sweeps (rtile.cu): k sweeps per launch, 1 <= k <= kRtMaxDepth (17 points: half)
+// register-tile FP32 sweeps (rtile.cu): k sweeps per launch, 1 <= k <= kRtMaxDepth (17 points: half).
+// r is read before the launch waits for the one before it, which must not write r (see above)
 cudaError_t launch_sweep32_rtile(const cj_plan *p, const float *e, const float *r, float *out,
                                  const float *w, int k, cudaStream_t s);
 // sweeps per launch with the shortest modelled time per sweep, for cycles of `sweeps` sweeps

@@ -184,8 +184,8 @@ __device__ __forceinline__ ff2 ff_side1(const FFRow &q) {
 __device__ __forceinline__ ff2 ff_side2(const FFRow &q) { return ff_add(ff2_of(q.l), ff2_of(q.r)); }
 
 // One weighted sweep out = u + w (L u - b): thread t has pair t mod np of chunk t / np, rows
-// chunk ty + 1 onwards.  Its launches overlap the end of the one before: nothing is read before
-// griddepcontrol.wait, which makes that sweep's stores visible.
+// chunk ty + 1 onwards.  Its launches overlap the end of the one before (programmatic dependent launch,
+// cj_internal.h).
 template <int ST>
 __global__ void __launch_bounds__(kFFThreads, ST == 17 ? 4 : 7) sweep_ff_kernel(const __grid_constant__ FFArgs a) {
     constexpr int R = ST == 17 ? 2 : 1;

@@ -36,10 +36,10 @@ __device__ __forceinline__ void rt_cp_async16(void *dst, const void *src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
 }
 
-// The launches of one inner cycle follow one another with programmatic dependent launch: a block
-// may start while the previous launch drains, stages r (which no sweep writes), and waits here for
-// that launch's end before it reads e or writes; only then may the launch after this one start.
-// (e is read past L1, which may still hold lines of the buffer from two launches earlier.)
+// The launches of one inner cycle follow one another with programmatic dependent launch (cj_internal.h):
+// a block may start while the previous launch drains, stages r (which no sweep writes, nor the launch
+// before a cycle's first), and waits here for that launch's end before it reads e or writes; only
+// then may the launch after this one start.  (e is read past L1: a block reads each node once.)
 __device__ __forceinline__ void rt_wait_previous() {
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");

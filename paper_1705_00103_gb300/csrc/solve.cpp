@@ -959,6 +959,7 @@ cj_status cj_sweeps_f32(cj_plan *p, const float *r, long long ldr, float *e, lon
     if (a != CJ_OK) return a;
     if (first < 0 || count < 0 || !p->e0) return CJ_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
+    // (r first: the sweeps' first launch may read it before it waits for the launch before)
     CJ_TRY(launch_import32(p, r, ldr, p->rt, s), "import32 r");
     CJ_TRY(launch_import32(p, e, lde, p->e0, s), "import32 e");
     float *cur = p->e0, *nxt = p->e1;

@@ -18,7 +18,7 @@
 //
 // A thread walks `ty` rows of one column, the next row's loads one iteration ahead; threads
 // number the columns of one chunk of rows after the other, so narrow grids leave no lane idle.
-// Sweeps follow one another with programmatic dependent launch (rtile_dev.cuh).
+// Sweeps follow one another with programmatic dependent launch (cj_internal.h).
 //
 // Measured on one GB300 (us per sweep; one 128-column block per strip with FP64 additions -> this):
 // 9-point 1001 x 701: 13.6 -> 8.5; 1024^2: 18.1 -> 11.5; 4096^2: 268 -> 138; 5-point 600 x 500: 5.2
@@ -79,7 +79,7 @@ struct S64Args {
     int k;
 };
 
-// Rows j0..j1 of column i.  u is read past L1, which may hold lines from two launches earlier.
+// Rows j0..j1 of column i.  (u is read past L1; through it, the sweep takes the same time.)
 template <int ST>
 __device__ __forceinline__ void march64(const S64Args &a, int i, int j0, int j1, double w) {
     using C = Co<double>;
