@@ -11,7 +11,7 @@
 // Engine tile: the unit of work of every engine kernel, kEngTX columns x (per slot) ty rows of
 // nodes; ty is 16, 32 (the default) or 64, chosen per stencil and size class by
 // cj_autotune_engine.
-constexpr int kEngTX = 128, kEngTYDefault = 32, kEngTYMax = 64;
+constexpr int kEngTX = 128, kEngTYDefault = 32;
 
 enum SlotPhase : int {
     PHASE_FREE = 0,     // unused

@@ -16,11 +16,6 @@ struct Ar<double> {
     }
     static __device__ __forceinline__ double fm(double a, double b, double c) { return fma(a, b, c); }
 };
-template <>
-struct Ar<float> {
-    static __device__ __forceinline__ float add(float a, float b, float) { return a + b; }
-    static __device__ __forceinline__ float fm(float a, float b, float c) { return fmaf(a, b, c); }
-};
 
 // Stencil coefficients of h^2 Delta_h (Table 3; Eq. 1 and Fig. 1 left; Eq. 2 and Fig. 1
 // right), rounded once to the working type.
@@ -37,18 +32,6 @@ struct Co<double> {
     static __device__ __forceinline__ double d1() { return 16.0 / 72.0; }
     static __device__ __forceinline__ double d2() { return -1.0 / 72.0; }
     static __device__ __forceinline__ double cc17() { return -300.0 / 72.0; }
-};
-template <>
-struct Co<float> {
-    static __device__ __forceinline__ float c5() { return -4.0f; }
-    static __device__ __forceinline__ float ax9() { return 4.0f / 6.0f; }
-    static __device__ __forceinline__ float dg9() { return 1.0f / 6.0f; }
-    static __device__ __forceinline__ float cc9() { return -20.0f / 6.0f; }
-    static __device__ __forceinline__ float a1() { return 64.0f / 72.0f; }
-    static __device__ __forceinline__ float a2() { return -4.0f / 72.0f; }
-    static __device__ __forceinline__ float d1() { return 16.0f / 72.0f; }
-    static __device__ __forceinline__ float d2() { return -1.0f / 72.0f; }
-    static __device__ __forceinline__ float cc17() { return -300.0f / 72.0f; }
 };
 
 template <typename T>
