@@ -437,7 +437,7 @@ def mixed_paths(cj, f, stream, fp64dd, peaks):
             r = cj.cj_solve(p.handle, f, u, stream)
             M_in = p.info()["M_inner"]
         upd_s = N_GRID * N_GRID * r["sweeps"] / r["sweep_seconds"]
-        k = depth if depth else 4
+        k = depth if depth else 8  # the default depth at this size (fp32_sweep_roofline)
         out[name] = {"time_s": r["seconds"], "rel_res_l2": r["rel_res_l2"], "status": cj.cj_status_string(r["rc"]),
                      "fp32_sweeps": r["sweeps"], "outer_steps": r["cycles"], "inner_cycle": M_in,
                      "temporal_depth": depth if depth else "auto (8 for this stencil and size unless "
@@ -454,7 +454,7 @@ def mixed_paths(cj, f, stream, fp64dd, peaks):
 
 def small_solve(cj, stream, runs: int = 5) -> dict:
     """The small case (5-point, 64 x 64, FP64, tol 1e-10, the sin*sin right-hand side): time to
-    tolerance of whole cj_solve calls (graph-launched cycles), median of `runs` after 3 warm-up
+    tolerance of whole cj_solve calls (one cluster launch each), median of `runs` after 3 warm-up
     solves; the call blocks until the solve ends, so host time is the time to tolerance."""
     import torch
     import workloads
@@ -1070,7 +1070,7 @@ def serve_key(cj, n_requests: int, fp64_every: int = 4, fp64_max_nodes: int = 1 
                                    "note": "every %d-th request of at most %d nodes, alone: plain FP64 CJM for tol "
                                            "1e-6, FP64 cycles in double-FP64 defect correction for 1e-10; for these "
                                            "small requests the FP64 path alone is faster than their service in the "
-                                           "mix, whose engine spends ~2.5 launches per sweep"
+                                           "mix, beside the other requests on the device"
                                            % (fp64_every, fp64_max_nodes)},
             "fp64_whole_prefix_lower_bound_s_extrapolated": lower,
             "speedup_vs_fp64_one_at_a_time_lower_bound": lower / wall,

@@ -106,10 +106,12 @@ typedef struct {
     long long max_sweeps;   /* sweep budget of one solve; 0 = 64 cycles (CJ_JACOBI: the larger
                                of 64 intervals and 4 ln(1/tol) / kmin sweeps) */
     int method;             /* cj_method (default CJ_CJM) */
-    int launch;             /* plain FP64 cycles: 0 = auto (a CUDA graph of the cycle's sweeps on
-                               grids of up to 2^22 nodes, where one sweep is shorter than a host
-                               launch; one launch per sweep above), 1 = one launch per sweep,
-                               2 = the graph at any size (needs an even M) */
+    int launch;             /* plain FP64 cycles: 0 = auto (the whole solve in one cluster of
+                               thread blocks on grids of up to 2^14 nodes where that is the fastest,
+                               a CUDA graph of the cycle's sweeps on grids of up to 2^22 nodes,
+                               where one sweep is shorter than a host launch, one launch per sweep
+                               above), 1 = one launch per sweep, 2 = the graph at any size (needs
+                               an even M), 3 = the cluster solve (up to 2^14 nodes) */
 } cj_options;
 
 /* What one solve did.  The relative residuals are those of the returned u:
@@ -381,15 +383,17 @@ typedef struct {
  * cj_solve_batch -- solve n independent problems (any sizes, stencils, tolerances) together
  * with the mixed-precision CJM: FP32 inner cycles inside FP64 or double-FP64 defect
  * correction, every problem's residual test and stop rule evaluated on the device.  The
- * problems run as slots of one engine whose step (correct, defect, decide, eight sweep
- * launches, export, advance: launches over persistent
- * grids that read a device tile list of 128-column tiles) is captured once in a CUDA graph
- * and replayed until every slot has finished; finished problems leave the tile list; tile
- * rows (16/32/64; of the outer steps' kernels) come from cj_autotune_engine's table for the size
- * class when it has an entry.  The sweeps run on register tiles, eight per launch (17 points:
- * four) unless the table or the problem names another depth, the problems of one stencil and tile shape in one branch of the step's graph.  A problem's arithmetic does not depend on its batch-mates.  results[k] receives problem k's outcome (status per
- * problem; seconds and launches are those of the whole batch).  Orders itself after the
- * work already on `stream` and makes `stream` wait for it; blocks until done.  Returns
+ * problems run as slots of one engine whose step (correct, defect, decide, 8, 16 or 32 sweep
+ * launches by the longest inner cycle, export, advance: launches over persistent grids that read
+ * device lists of tiles) is captured once in a CUDA graph and replayed until every slot has
+ * finished; finished problems leave the lists; tile rows (16/32/64; of the outer steps' kernels)
+ * come from cj_autotune_engine's table for the size class when it has an entry.  The sweeps run on
+ * register tiles, eight per launch (17 points: four) unless the table or the problem names another
+ * depth (depth 1 of 5 and 9 points: on the 128-column tiles), the problems of one stencil and tile
+ * shape in one branch of the step's graph.  A problem's arithmetic does not depend on its
+ * batch-mates.  results[k] receives problem k's outcome (status per problem; seconds and launches
+ * are those of the whole batch).  Orders itself after the work already on `stream` and makes
+ * `stream` wait for it; blocks until done.  Returns
  * CJ_OK, or CJ_ERR_TIMEOUT if a problem did not finish within its sweep budget's steps.
  */
 cj_status cj_solve_batch(const cj_problem *problems, int n, void *stream, cj_result *results);

@@ -18,7 +18,7 @@
 //   advance  -- per slot: move the cycle counter and the ping-pong by the step's sweeps,
 //               retire exported slots, publish a compact status record for the host.
 // The launches read the tile list and the slots' phases from device memory, so a CUDA graph
-// of many steps is captured once and replayed unchanged while problems come and go.  No
+// of a step is captured once and replayed unchanged while problems come and go.  No
 // kernel waits on another block: every dependency is a kernel boundary.
 //
 // Per node, every kernel evaluates the same arithmetic, in the same order, as the

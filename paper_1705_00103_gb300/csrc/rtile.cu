@@ -3,8 +3,8 @@
 // Measured on one GB300 (us per sweep, one sweep per launch or the per-warp row wavefront these
 // tiles replaced -> tiles at their default depth): 9-point 333 x 250: 3.9 -> 0.44; 1023^2: 3.8 ->
 // 0.94; 4096^2: 13.9 -> 9.2 (1834 Gupd/s); 8192^2: 45 -> 32.7 (2053 Gupd/s); 17-point 8192^2:
-// 159 -> 68.8 (976 Gupd/s); 400^2: 4.0 -> 1.2.  On large grids the FMA pipe is busy 67 % of the
-// cycles (9.25 operations per node and sweep for 9 points, times the tile's overlap of 1.33); the
+// 159 -> 68.8 (976 Gupd/s); 400^2: 4.0 -> 1.2.  On large grids the FMA pipe is busy 66 % of an SM's
+// cycles (4096^2; 9.25 operations per node and sweep for 9 points, times the tile's overlap of 1.34); the
 // rest is the loads and stores at the ends of a tile's life, which the other block of the SM hides
 // only in part.  On small ones the launch and the tile's load and store (2.3 us together, with
 // programmatic dependent launch) stand beside k sweeps of a quarter of a microsecond each.

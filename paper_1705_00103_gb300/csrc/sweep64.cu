@@ -20,10 +20,13 @@
 // number the columns of one chunk of rows after the other, so narrow grids leave no lane idle.
 // Sweeps follow one another with programmatic dependent launch (cj_internal.h).
 //
-// Measured on one GB300 (us per sweep; one 128-column block per strip with FP64 additions -> this):
-// 9-point 1001 x 701: 13.6 -> 8.5; 1024^2: 18.1 -> 11.5; 4096^2: 268 -> 138; 5-point 600 x 500: 5.2
-// -> 4.1; 1024^2: 13.2 -> 8.8; 4096^2: 216 -> 114; 17-point 129 x 200: 4.1 -> 3.0; 1000 x 1100: 33.2
-// -> 23.9; 4096^2: 475 -> 287.
+// Measured on one GB300 (us per sweep; one 128-column block per strip with FP64 additions -> this) on
+// smooth iterates: 9-point 1001 x 701: 13.6 -> 8.5; 1024^2: 18.1 -> 11.5; 4096^2: 268 -> 134; 5-point
+// 600 x 500: 5.2 -> 4.1; 1024^2: 13.2 -> 8.8; 4096^2: 216 -> 112; 17-point 129 x 200: 4.1 -> 3.0; 1000 x
+// 1100: 33.2 -> 23.9; 4096^2: 475 -> 276.  An iterate with a sign change in every warp's row, or of
+// zeros, gains little (noise or zeros, 4096^2: 9-point 268 -> 248, 5-point 216 -> 187, 17-point 475 -> 466);
+// others lie between (16 9-point sweeps of 4096^2 that smooth a rough iterate, with import and export:
+// 4.67 -> 4.07 ms).
 #include "cj_internal.h"
 #include "grid_dev.cuh"
 #include "stencil_dev.cuh"

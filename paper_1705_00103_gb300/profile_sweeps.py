@@ -6,9 +6,9 @@
     python -m paper_1705_00103_gb300.profile_sweeps --stencil 9 --n 4096 --precision ff --count 16
     python -m paper_1705_00103_gb300.profile_sweeps --stencil 9 --n 1024 --batch 24 --depth 4
 
-Inputs are zero grids of the given size (FP64 sweeps of them take every row's additions on the FP64
-pipe: twice the time of a smooth iterate; the others' cost does not depend on the values);
-three FP64 grids of 4096^2 (400 MB) exceed the 129 MB L2.
+Inputs are zero grids of the given size, or a smooth iterate (--iterate smooth: u = x (1 - x) y (1 - y),
+f = -1) or a rough one (normal noise).  FP64 sweeps of zero grids take every row's additions on the FP64
+pipe: twice the time of a smooth iterate; the others' cost does not depend on the values.  Three FP64 grids of 4096^2 (400 MB) exceed the 129 MB L2.
 """
 from __future__ import annotations
 
@@ -25,6 +25,8 @@ def main(argv=None):
     ap.add_argument("--n", type=int, default=4096)
     ap.add_argument("--precision", default="fp64", choices=["fp64", "fp32", "ff"],
                     help="ff: the FP64 sweep in float-float on the FP32 pipe (cj_sweeps_ff)")
+    ap.add_argument("--iterate", default="zero", choices=["zero", "smooth", "rough"],
+                    help="FP64 and float-float sweeps: what they start from")
     ap.add_argument("--count", type=int, default=3)
     ap.add_argument("--depth", type=int, default=1, help="FP32 sweeps per launch (temporal blocking)")
     ap.add_argument("--time", type=int, default=0,
@@ -87,6 +89,12 @@ def main(argv=None):
         with cj.Plan(a.n, a.n, a.stencil, 1e-10) as p:
             f = torch.zeros((a.n, a.n), dtype=torch.float64, device="cuda")
             u = torch.zeros_like(f)
+            if a.iterate == "smooth":
+                x = torch.arange(1, a.n + 1, dtype=torch.float64, device="cuda") / (a.n + 1)
+                u += (x * (1 - x))[:, None] * (x * (1 - x))
+                f -= 1.0
+            elif a.iterate == "rough":
+                u.normal_(generator=torch.Generator(device="cuda").manual_seed(1))
             run(lambda c: sweeps(p.handle, f, u, 0, c))
     else:
         with cj.Plan(a.n, a.n, a.stencil, 1e-10, precision=cj.CJ_FP32_INNER, temporal_depth=a.depth) as p:
