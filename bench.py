@@ -1056,7 +1056,7 @@ def serve_key(cj, n_requests: int, fp64_every: int = 4, fp64_max_nodes: int = 1 
     return {"workload": "served: arrival-faithful prefix of the seeded Poisson stream (2000/s), first %d of "
                         "10,000 requests, sides log-uniform in [32, 8192], 5/9/17-point, tol 1e-6 / 1e-10, "
                         "budget 150 GB" % len(reqs),
-            "requests": len(reqs), "full_stream": "10,000 requests: not run (about 80x the GPU's throughput "
+            "requests": len(reqs), "full_stream": "10,000 requests: not run (about 60x the GPU's throughput "
                                                  "over its 5 s arrival window)",
             "latency_s": {"p50": float(np.percentile(lat, 50)), "p99": float(np.percentile(lat, 99)),
                           "max": float(max(lat))},
